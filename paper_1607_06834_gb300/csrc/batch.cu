@@ -124,6 +124,7 @@ void group_consts(const rok_problem_desc &d, StencilConsts &C)
     C.gg = C.inv_gm1 + 1.0;
     C.gm1h = 0.5 * C.gm1;
     C.efix_k = (1.0 - C.efix) / (1.0 + C.efix);
+    set_fixed_consts(C);
 }
 
 // instances of one group share the gas model and scheme constants
@@ -381,6 +382,7 @@ rok_status rok_batch_init(rok_batch **out, const rok_problem_desc *descs, int co
         I.hrdy = 0.5 * I.rdy;
         if (d.kind == ROK_NS2D)
             face_coefs(I.mu, d.sutherland_s > 0.0, d.gamma / ((d.gamma - 1.0) * d.prandtl), I.rdx, I.rdy, I.vk);
+        set_fixed_visc(I.vk, d.sutherland_s > 0.0 ? I.mu : 1.0, I.fxv);
         off += (size_t)I.nchunks * kChunk;
         chunk += I.nchunks;
         for (int c = 0; c < I.nchunks; ++c) chunk_inst.push_back(k);

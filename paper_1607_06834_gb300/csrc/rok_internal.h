@@ -2,6 +2,7 @@
 // drivers and the kernels, launch helpers, status codes on the device.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -19,6 +20,27 @@ enum : int {
     kStatusTimeout = 4,    // a bounded device wait (arrival counter) gave up
 };
 
+
+// Constants of the fixed-point stencil (FMA build, stencil_fixed.cuh): numbers
+// x 2^(62 - S), S the scale in the name's comment, and the bounds of the Mach
+// number |M| 2^26 between which Harten's fix acts.
+struct FixedConsts {
+    int ok;                    // the gas model and scheme constants are in the formats' ranges
+    int m_lo, m_hi;            // (1 - efix) / (1 + efix) and its inverse
+    int fix_ok;                // efix in the range of the fix's fixed-point form
+    long long efix, hfix;      // efix (0), 1 / (2 efix) (3)
+    long long c_lo, c_hi;      // 0
+    long long gg, gm1;         // 3, 0
+    long long suth_s, suth_1s; // s / 4 (0), 1 + s (1)
+    long long itref;           // 1 / t_ref = itref 2^(itref_e - 62), mantissa in [1/2, 1)
+    int itref_e;
+};
+
+// Viscous coefficients vk as mantissas below 1/2 with one exponent: vk = k 2^(e - 62)
+struct FixedVisc {
+    long long k[2][5];
+    int e;
+};
 
 // Constants of the finite-volume residual (Sec. 3.2).  Every derived constant is
 // computed on the host by the same expression the plain CPU evaluation uses, so the
@@ -42,6 +64,8 @@ struct StencilConsts {
     double gg, gm1h, hrdx, hrdy;
     double vk[2][5];
     double vc[4];
+    FixedConsts fx;
+    FixedVisc fxv;
     double efix_k;             // (1 - efix) / (1 + efix): c~ efix_k >= |u~| <=> c~ - |u~| >= efix (|u~| + c~)
 };
 
@@ -68,6 +92,51 @@ inline void face_coefs(double mu, bool sutherland, double kfac, double rdx, doub
     }
 }
 
+// the mantissas of factor vk (nothing finite: an exponent no state's units reach)
+inline void set_fixed_visc(const double vk[2][5], double factor, FixedVisc &V)
+{
+    double m = 0.0;
+    for (int d = 0; d < 2; ++d)
+        for (int q = 0; q < 5; ++q) {
+            const double a = fabs(factor * vk[d][q]);
+            m = a > m || !(a == a) ? a : m;
+        }
+    const bool zero = m == 0.0, finite = m < 1e300 && m > 1e-300;
+    int x = 0;
+    if (finite) frexp(m, &x);
+    V.e = zero ? -2000 : (finite ? x + 1 : 1 << 20);
+    for (int d = 0; d < 2; ++d)
+        for (int q = 0; q < 5; ++q) V.k[d][q] = finite ? (long long)ldexp(factor * vk[d][q], 62 - V.e) : 0;
+}
+
+// the fixed-point constants from the gas model and scheme constants (gm1, gg, c_lo,
+// c_hi, efix, inv_tref, suth_s)
+template <class Consts>
+inline void set_fixed_consts(Consts &C)
+{
+    FixedConsts &F = C.fx;
+    F = FixedConsts{};
+    F.ok = C.gm1 >= 0.2 && C.gm1 < 1.0 && C.gg <= 6.0 && fabs(C.c_lo) < 1.0 && fabs(C.c_hi) < 1.0 && C.efix >= 0.0 &&
+           C.efix < 1.0;
+    if (C.sutherland) F.ok = F.ok && C.suth_s > 0.0 && C.suth_s < 1.0 && C.inv_tref > 1e-300 && C.inv_tref < 1e300;
+    if (!F.ok) return;
+    const double lo = (1.0 - C.efix) / (1.0 + C.efix), hi = (1.0 + C.efix) / (1.0 - C.efix);
+    F.m_lo = (int)ldexp(lo, 26);
+    F.m_hi = (int)ceil(ldexp(hi < 31.0 ? hi : 31.0, 26));
+    F.fix_ok = C.efix > 0.0625 && C.efix <= 1.0 / 3.0;
+    F.efix = (long long)ldexp(C.efix, 62);
+    F.hfix = F.fix_ok ? (long long)ldexp(0.5 / C.efix, 59) : 0;
+    F.c_lo = (long long)ldexp(C.c_lo, 62);
+    F.c_hi = (long long)ldexp(C.c_hi, 62);
+    F.gg = (long long)ldexp(C.gg, 59);
+    F.gm1 = (long long)ldexp(C.gm1, 62);
+    if (C.sutherland) {
+        F.suth_s = (long long)ldexp(C.suth_s, 60);
+        F.suth_1s = (long long)ldexp(1.0 + C.suth_s, 61);
+        F.itref = (long long)ldexp(frexp(C.inv_tref, &F.itref_e), 62);
+    }
+}
+
 // the FMA-build constants from the fields above (gm1, inv_gm1, mu, kfac, rdx, rdy)
 inline void set_fast_consts(StencilConsts &C)
 {
@@ -82,6 +151,8 @@ inline void set_fast_consts(StencilConsts &C)
     C.vc[1] = -m * (2.0 / 3.0);
     C.vc[2] = m;
     C.vc[3] = m * C.kfac;
+    set_fixed_consts(C);
+    set_fixed_visc(C.vk, C.sutherland ? C.mu : 1.0, C.fxv);
 }
 
 // Face metrics of a curvilinear grid (device arrays).
@@ -131,6 +202,7 @@ struct BatchInst {
     int chunk0, nchunks;       // first 2048-entry chunk and chunk count P_k
     double rdx, rdy, q_rdx, q_rdy, mu;
     double hrdx, hrdy, vk[2][5];   // FMA-build constants (face_coefs)
+    FixedVisc fxv;
 };
 
 // Tile table of one batched stencil launch (device arrays): CTA b computes tile

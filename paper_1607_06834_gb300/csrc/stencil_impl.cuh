@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "dual.cuh"
+#include "fixed.cuh"
 #include "rok_internal.h"
 
 namespace rok {
@@ -36,7 +37,7 @@ namespace ROK_NS {
 template <int TXv, int TYv, int NTv = TXv * TYv>
 struct Shape {
     static constexpr int TX = TXv, TY = TYv, NT = NTv, EW = TXv + 4, EH = TYv + 4;
-    static_assert((TXv * TYv) % NTv == 0, "whole cells per thread");
+
 };
 using Shape32x8 = Shape<32, 8>;
 using CurvShape = Shape<16, 16>;
@@ -880,6 +881,10 @@ __global__ void __launch_bounds__(CartShape::NT, MINB) cart_kernel(const Stencil
     cart_tile<VISC, SUTH, S, CartShape>(C, io, blockIdx.x * CartShape::TX, blockIdx.y * CartShape::TY, smem_raw);
 }
 
+#ifdef ROK_STENCIL_FAST
+#include "stencil_fixed.cuh"
+#endif
+
 // Many independent uniform periodic grids of one physics group in one launch:
 // CTA b computes tile b - tile_first[k] of instance k = tile_inst[b].  The
 // instances share the gas model and scheme constants (C); grid size, spacing
@@ -1255,6 +1260,38 @@ static cudaError_t launch_cart_t(const StencilConsts &c, const StencilIO &io, cu
     return cudaGetLastError();
 }
 
+#ifdef ROK_STENCIL_FAST
+template <bool V, bool SU, class SH>
+static cudaError_t launch_fixed_tiles(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
+{
+    const size_t smem = FixedSmem<SU, SH>::bytes;
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(fixed_cart_kernel<V, SU, SH, kFixedMinB>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    dim3 grid((c.nx + SH::TX - 1) / SH::TX, (c.ny + SH::TY - 1) / SH::TY);
+    fixed_cart_kernel<V, SU, SH, kFixedMinB><<<grid, SH::NT, smem, s>>>(c, io);
+    return cudaGetLastError();
+}
+
+// The tile by the grid's size (the bits do not depend on it).  FD-JVP, viscous,
+// us a launch, 16 x 7 / 16 x 16 / 32 x 15: 128^2 10.3 / 16.4 / 24.6 (the
+// grid is below one CTA per SM: the smallest chain of rounds wins); 512^2
+// 63.5 / 59.7 / 60.8; 1024^2 264 / 224 / 205 (32 x 15 loads 1.43 cells a cell
+// where 16 x 16 loads 1.56, but needs three full waves of 3 CTAs per SM).
+template <bool V, bool SU>
+static cudaError_t launch_fixed_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
+{
+    auto tiles = [&](int tx, int ty) { return (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty); };
+    if (tiles(32, 15) >= 3 * 3 * 152) return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
+    if (tiles(16, 16) > 152) return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
+    return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
+}
+#endif
+
 template <bool V, bool SU, class S>
 static cudaError_t launch_curv_t(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
 {
@@ -1277,6 +1314,12 @@ static cudaError_t launch_curv_t(const StencilConsts &c, const CurvGeom &g, cons
 cudaError_t launch_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
     const bool dual = io.dir || io.dirf;
+#ifdef ROK_STENCIL_FAST
+    if (!dual && c.fx.ok) {
+        if (!c.viscous) return launch_fixed_cart<false, false>(c, io, s);
+        return c.sutherland ? launch_fixed_cart<true, true>(c, io, s) : launch_fixed_cart<true, false>(c, io, s);
+    }
+#endif
     if (!c.viscous) return dual ? launch_cart_t<false, false, Dual>(c, io, s) : launch_cart_t<false, false, double>(c, io, s);
     if (c.sutherland)
         return dual ? launch_cart_t<true, true, Dual>(c, io, s) : launch_cart_t<true, true, double>(c, io, s);
@@ -1287,6 +1330,21 @@ template <bool V, bool SU, class SH>
 static cudaError_t launch_cart_batch_t(const StencilConsts &c, const StencilIO &io, const BatchTiles &bt, int ntiles,
                                        cudaStream_t s)
 {
+#ifdef ROK_STENCIL_FAST
+    if (c.fx.ok) {
+        typedef FixedShape<SH> FS;
+        const size_t smem = FixedSmem<SU, FS>::bytes;
+        static bool attr_set = false;
+        if (!attr_set) {
+            cudaError_t e = cudaFuncSetAttribute(fixed_batch_kernel<V, SU, FS, kFixedMinB>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            attr_set = true;
+        }
+        fixed_batch_kernel<V, SU, FS, kFixedMinB><<<ntiles, FS::NT, smem, s>>>(c, io, bt);
+        return cudaGetLastError();
+    }
+#endif
     const size_t smem = sizeof(Tile<double, SH>) + sizeof(Faces<double, SH>) + sizeof(Diffs<double, SH>) +
                         pair_sums_bytes<V, double, SH>();
     static bool attr_set = false;
