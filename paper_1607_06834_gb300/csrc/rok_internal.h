@@ -32,6 +32,7 @@ struct FixedConsts {
     long long c_lo, c_hi;      // 0
     long long gg, gm1;         // 3, 0
     long long suth_s, suth_1s; // s / 4 (0), 1 + s (1)
+    long long g_inf;           // mu / mu_ref of the free stream (2; negative: out of range)
     long long itref;           // 1 / t_ref = itref 2^(itref_e - 62), mantissa in [1/2, 1)
     int itref_e;
 };
@@ -133,6 +134,8 @@ inline void set_fixed_consts(Consts &C)
     if (C.sutherland) {
         F.suth_s = (long long)ldexp(C.suth_s, 60);
         F.suth_1s = (long long)ldexp(1.0 + C.suth_s, 61);
+        const double g = C.prim_inf[5] / C.mu;
+        F.g_inf = g >= 0.0 && g < 2.0 ? (long long)ldexp(g, 60) : -1;
         F.itref = (long long)ldexp(frexp(C.inv_tref, &F.itref_e), 62);
     }
 }
@@ -152,11 +155,22 @@ inline void set_fast_consts(StencilConsts &C)
     C.vc[2] = m;
     C.vc[3] = m * C.kfac;
     set_fixed_consts(C);
-    set_fixed_visc(C.vk, C.sutherland ? C.mu : 1.0, C.fxv);
+    const double curv[2][5] = {{C.vc[0], C.vc[1], C.vc[2], C.vc[3], 0.0}, {}};
+    set_fixed_visc(C.rdx > 0.0 ? C.vk : curv, C.sutherland ? C.mu : 1.0, C.fxv);   // rdx: 0 on curvilinear grids
 }
+
+// Fixed-point metrics of one face (64 bytes, read as four 16-byte words): the
+// unit normal, the diamond coefficients (c1, c3: a quarter, for four-cell
+// differences) as mantissas, c = mantissa 2^(e - 62), and half the face length
+struct alignas(16) FixedMetric {
+    long long nx, ny, c0, c1, c2, c3;
+    double hlen;
+    long long e;
+};
 
 // Face metrics of a curvilinear grid (device arrays).
 struct CurvGeom {
+    const FixedMetric *fi, *fj;   // FMA build: the faces' fixed-point metrics (same indices)
     // i-faces: (nx+1) * ny, index j*(nx+1)+i ; j-faces: nx * (ny+1), index j*nx+i
     const double *in_x, *in_y, *il, *ic0, *ic1, *ic2, *ic3;
     const double *jn_x, *jn_y, *jl, *jc0, *jc1, *jc2, *jc3;
@@ -222,6 +236,10 @@ inline int shape_ty(int s) { return s == kShape16x16 ? 16 : (s == kShape64x4 ? 4
 
 // stencil launchers, one set per rounding mode (separate translation units)
 namespace fast {
+// FMA build: the fixed-point metrics of n faces from their device arrays
+cudaError_t launch_fixed_metrics(const double *nx, const double *ny, const double *len, const double *c0,
+                                 const double *c1, const double *c2, const double *c3, size_t n, FixedMetric *out,
+                                 cudaStream_t s);
 cudaError_t launch_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s);
 cudaError_t launch_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s);
 cudaError_t launch_lorenz(const StencilConsts &c, const StencilIO &io, int n, cudaStream_t s);

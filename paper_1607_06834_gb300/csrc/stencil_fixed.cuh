@@ -164,6 +164,8 @@ struct FixedState {
 // a plain mul62 and results are realigned by shifts (a product that keeps more
 // bits costs five instructions more); the comments give the bounds that keep
 // the values in their formats.
+// ROUND: the uniform grids' roundings of the pressure sums.
+template <bool ROUND>
 __device__ __forceinline__ void fixed_roe(const FixedState &L, const FixedState &R, const FixedConsts &F, fx::Fx<0> vn,
                                           fx::Fx<0> vt, fx::Fx<0> ve, fx::Fx<0> (&G)[4], bool &bad)
 {
@@ -231,7 +233,8 @@ __device__ __forceinline__ void fixed_roe(const FixedState &L, const FixedState 
     if (outside<1>(Dn) || outside<1>(Dt) || outside<1>(D3)) bad = true;
     const Fx<0> mL = mul<0>(L.r, L.n), mR = mul<0>(R.r, R.n);   // below 1/2
     G[0] = (mL + mR) - D0;
-    G[1] = mul<0>(mL, L.n) + round53(mul<0>(mR, R.n) + round53(to<0>(round53(L.p + R.p)) - Dn));
+    if (ROUND) G[1] = mul<0>(mL, L.n) + round53(mul<0>(mR, R.n) + round53(to<0>(round53(L.p + R.p)) - Dn));
+    else G[1] = mul<0>(mL, L.n) + (mul<0>(mR, R.n) + (to<0>(L.p + R.p) - Dn));
     G[2] = mul<0>(mL, L.t) + (mul<0>(mR, R.t) - Dt);
     G[3] = mul<0>(L.n, eL) + (mul<0>(R.n, eR) - D3);
 }
@@ -412,7 +415,7 @@ __device__ __forceinline__ void fixed_cart_tile(const StencilConsts &C, const Gr
             }
             if (flag & 1) bad = true;
             Fx<0> G[4];
-            fixed_roe(L, R, F, vn, vt, ve, G, bad);
+            fixed_roe<true>(L, R, F, vn, vt, ve, G, bad);
             if (!bad) {
                 double *out = yd ? &fc.fy[0][fy][fx_] : &fc.fx[0][fy][fx_];
                 const int ks = yd ? (TY + 1) * TX : TY * (TX + 1);
@@ -475,4 +478,371 @@ __global__ void __launch_bounds__(SH::NT, MINB)
     const int ntx = (I.nx + SH::TX - 1) / SH::TX;
     fixed_cart_tile<VISC, SUTH, SH>(C, GridRef{I.nx, I.ny, I.hrdx, I.hrdy, I.mu}, I.fxv, I.vk, io, (t % ntx) * SH::TX,
                                     (t / ntx) * SH::TY, smem_raw, I.off, (size_t)k * bt.stride_bytes);
+}
+
+// ============================== curvilinear grid ===============================
+// The same for curv_kernel's grids.  A face's reconstructed velocities are
+// rotated into its (normal, tangential) frame, fixed_roe runs there (the flux is
+// invariant under rotation) and the momentum fluxes are rotated back: twelve
+// products more than the uniform faces.  The normals are 62-bit fractions; the
+// diamond coefficients of a face are mantissas with one exponent per face
+// (they span the inverse cell widths, 1e-2 to 1e4 on a stretched grid), which
+// the viscous terms are shifted by.  Residual on the 256 x 512 O-grid with
+// Sutherland's law: 134 -> 45 us.
+
+__device__ __forceinline__ FixedMetric fixed_metric(double nx, double ny, double len, double c0, double c1, double c2,
+                                                    double c3)
+{
+    const auto unit = [](double x) {   // |x| <= 1 in 62 bits, 1 just below
+        const long long one = 1ll << 62, v = (long long)(x * 4611686018427387904.0);
+        return v >= one ? one - 1 : (v <= -one ? 1 - one : v);
+    };
+    FixedMetric m{unit(nx), unit(ny), 0, 0, 0, 0, 0.5 * len, 1 << 20};
+    const double c[4] = {c0, 0.25 * c1, c2, 0.25 * c3};
+    double big = 0.0;
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        big = fmax(big, fabs(c[k]));
+        ok = ok && isfinite(c[k]);
+    }
+    const int x = (__double2hiint(big) >> 20) - 1022;   // big in [2^(x-1), 2^x)
+    if (!ok || x < -900 || x > 900) return m;             // an exponent no state's units reach
+    m.e = x + 1;
+    const double up = pow2(62 - x - 1);
+    m.c0 = (long long)(c[0] * up);
+    m.c1 = (long long)(c[1] * up);
+    m.c2 = (long long)(c[2] * up);
+    m.c3 = (long long)(c[3] * up);
+    return m;
+}
+
+// x 2^l for l in [0, 30]; bad where it would reach 1/2
+__device__ __forceinline__ fx::Fx<0> scale_up(fx::Fx<0> x, int l, bool &bad)
+{
+    const int top = (int)(x.v >> 31) >> (30 - l);   // 0 or -1 where 2^l x stays below 1/2
+    if (top != 0 && top != -1) bad = true;
+    return {(long long)((unsigned long long)x.v << l)};
+}
+
+// ghost rules of one tile cell (global indices gi, gj): the source cell, whether
+// its velocity is mirrored, whether it is the free stream
+__device__ __forceinline__ void curv_source(const StencilConsts &C, int &gi, int &gj, bool &mirror, bool &inf)
+{
+    const int nx = C.nx, ny = C.ny;
+    mirror = inf = false;
+    if (gi < 0 || gi >= nx) {
+        const int b = gi < 0 ? C.bc[0] : C.bc[1];
+        if (b == ROK_BC_PERIODIC) gi = wrapi(gi, nx);
+        else if (b == ROK_BC_WALL) { gi = gi < 0 ? -gi - 1 : 2 * nx - 1 - gi; mirror = !mirror; }
+        else inf = true;
+    }
+    if (!inf && (gj < 0 || gj >= ny)) {
+        const int b = gj < 0 ? C.bc[2] : C.bc[3];
+        if (b == ROK_BC_PERIODIC) gj = wrapi(gj, ny);
+        else if (b == ROK_BC_WALL) { gj = gj < 0 ? -gj - 1 : 2 * ny - 1 - gj; mirror = !mirror; }
+        else inf = true;
+    }
+    // a tile cell past the last valid index of a partial tile may still be out of
+    // range after the rules above; clamp it (its faces are never used)
+    gi = min(max(gi, 0), nx - 1);
+    gj = min(max(gj, 0), ny - 1);
+}
+
+// the faces left out by the fixed-point path, in binary64 (as slow_faces)
+template <bool VISC, bool SUTH, class SH>
+__device__ __noinline__ void slow_curv_faces(const StencilConsts &C, const CurvGeom &G, const StencilIO &io, int i0,
+                                             int j0, unsigned char *smem_raw, Faces<double, SH> &fc,
+                                             const FixedShared &fs, const unsigned *slow)
+{
+    constexpr int TX = SH::TX, TY = SH::TY, NT = SH::NT, EW = SH::EW, EH = SH::EH;
+    typedef double Arr[EH][EW];
+    Arr *w = reinterpret_cast<Arr *>(smem_raw);   // rho, u, v, p, T, mu
+    const int nx = C.nx, tid = threadIdx.x;
+    const size_t nc = (size_t)nx * C.ny;
+    double cf[kMaxAdd], cff, s1, s2;
+    coefs(io, cf, cff, s1, s2);
+    __syncthreads();
+    for (int idx = tid; idx < EW * EH; idx += NT) {
+        const int lx = idx % EW, ly = idx / EW;
+        int gi = i0 + lx - 2, gj = j0 + ly - 2;
+        bool mirror, inf;
+        curv_source(C, gi, gj, mirror, inf);
+        double q[6];
+        if (inf) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) q[k] = C.prim_inf[k];
+        } else {
+            const size_t c = (size_t)gj * nx + gi;
+            const double rho = load_value(io, cf, cff, c), mx = load_value(io, cf, cff, nc + c);
+            const double my = load_value(io, cf, cff, 2 * nc + c), E = load_value(io, cf, cff, 3 * nc + c);
+            const double rinv = rcp(rho);
+            q[0] = rho;
+            q[1] = mx * rinv;
+            q[2] = my * rinv;
+            q[3] = C.gm1 * E - C.gm1h * (mx * q[1] + my * q[2]);
+            q[4] = q[3] * rinv;
+            if (SUTH) {
+                const double tt = q[4] * C.inv_tref;
+                q[5] = C.mu * (tt * sqrt(tt)) * ((1.0 + C.suth_s) / (tt + C.suth_s));
+            }
+        }
+        w[0][ly][lx] = q[0];
+        w[1][ly][lx] = mirror ? -q[1] : q[1];
+        w[2][ly][lx] = mirror ? -q[2] : q[2];
+        w[3][ly][lx] = q[3];
+        w[4][ly][lx] = q[4];
+        if (SUTH) w[SUTH ? 5 : 0][ly][lx] = q[5];
+    }
+    __syncthreads();
+    constexpr int NFX_ = (TX + 1) * TY, NF = NFX_ + TX * (TY + 1);
+    for (int f = tid; f < NF; f += NT) {
+        if (!(slow[f >> 5] >> (f & 31) & 1)) continue;
+        const bool yd = f >= NFX_;
+        const int g = yd ? f - NFX_ : f;
+        const int fx = yd ? g % TX : g % (TX + 1), fy = yd ? g / TX : g / (TX + 1);
+        const int gi = i0 + fx, gj = j0 + fy;
+        const size_t fi = yd ? (size_t)gj * nx + gi : (size_t)gj * (nx + 1) + gi;
+        const int ym = yd ? fy + 1 : fy + 2, xm = yd ? fx + 2 : fx + 1, yp = fy + 2, xp = fx + 2;
+        const int sy = yp - ym, sx = xp - xm;            // unit step along the normal
+        const int ty = yd ? 0 : 1, txo = yd ? -1 : 0;    // tangential step
+        double WL[4], WR[4], Fl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            muscl(w[k][ym - sy][xm - sx], w[k][ym][xm], w[k][yp][xp], w[k][yp + sy][xp + sx], C.c_lo, C.c_hi, WL[k],
+                  WR[k]);
+        const double nxf = yd ? G.jn_x[fi] : G.in_x[fi], nyf = yd ? G.jn_y[fi] : G.in_y[fi];
+        double v1 = 0.0, v2 = 0.0, v3 = 0.0;
+        if (VISC) {
+            auto across = [&](const Arr &a) { return a[yp][xp] - a[ym][xm]; };
+            auto along = [&](const Arr &a) {
+                return (a[ym + ty][xm + txo] + a[yp + ty][xp + txo]) - (a[ym - ty][xm - txo] + a[yp - ty][xp - txo]);
+            };
+            visc_n2_terms<SUTH>(nxf, nyf, yd ? G.jc0[fi] : G.ic0[fi], quarter(yd ? G.jc1[fi] : G.ic1[fi]),
+                                yd ? G.jc2[fi] : G.ic2[fi], quarter(yd ? G.jc3[fi] : G.ic3[fi]), across(w[1]),
+                                across(w[2]), across(w[4]), along(w[1]), along(w[2]), along(w[4]),
+                                w[1][ym][xm] + w[1][yp][xp], w[2][ym][xm] + w[2][yp][xp],
+                                SUTH ? w[SUTH ? 5 : 0][ym][xm] + w[SUTH ? 5 : 0][yp][xp] : 0.0, C, v1, v2, v3);
+        }
+        roe_n2<VISC>(WL, WR, nxf, nyf, C, Fl, v1, v2, v3);
+        const double len = half(yd ? G.jl[fi] : G.il[fi]);
+        double *out = yd ? &fc.fy[0][fy][fx] : &fc.fx[0][fy][fx];
+        const int ks = yd ? (TY + 1) * TX : TY * (TX + 1);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[k * ks] = (Fl[k] * len) * fs.up[k];
+    }
+}
+
+template <bool VISC, bool SUTH, class SH, int MINB>
+__global__ void __launch_bounds__(SH::NT, MINB)
+    fixed_curv_kernel(const __grid_constant__ StencilConsts C, const __grid_constant__ CurvGeom G,
+                      const __grid_constant__ StencilIO io)
+{
+    using namespace fx;
+    constexpr int TX = SH::TX, TY = SH::TY, NT = SH::NT, EW = SH::EW, EH = SH::EH;
+    constexpr int NFX_ = (TX + 1) * TY, NF = NFX_ + TX * (TY + 1);
+    if (io.active && *io.active == 0) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ FixedShared fs;
+    __shared__ unsigned slow[(NF + 31) / 32];
+    __shared__ long long winf[6];
+    typedef FixedTile<SUTH, SH> FT;
+    FT &tl = *reinterpret_cast<FT *>(smem_raw);
+    Faces<double, SH> &fc = *reinterpret_cast<Faces<double, SH> *>(smem_raw + FixedSmem<SUTH, SH>::faces);
+    const FixedConsts &F = C.fx;
+    const int nx = C.nx, ny = C.ny;
+    const size_t nc = (size_t)nx * ny;
+    const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
+    const int tid = threadIdx.x;
+    double cf[kMaxAdd], cff, s1, s2;
+    coefs(io, cf, cff, s1, s2);
+    int eR, eU;
+    fixed_scales(io.base[0], io.base[3 * nc], eR, eU);
+    if (tid < 4) {
+        const int e = eR + eU * (tid == 0 ? 1 : (tid == 3 ? 3 : 2)) - 62;
+        fs.bx[tid] = pow2(e);
+        fs.up[tid] = pow2(-e);
+    }
+    if (tid == 32) {   // the free stream (far-field ghosts)
+        fs.any_slow = 0;
+        bool bad = false;
+        const Fx<0> r = from_double<0>(C.prim_inf[0], eR, bad), u = from_double<0>(C.prim_inf[1], eU, bad);
+        const Fx<0> v = from_double<0>(C.prim_inf[2], eU, bad), T = from_double<0>(C.prim_inf[4], 2 * eU, bad);
+        const Fx<-3> p = from_double<-3>(C.prim_inf[3], eR + 2 * eU, bad);
+        if (!in_window<4>(r) || !in_window<8>(p) || outside<1>(u) || outside<1>(v) || outside<1>(T)) bad = true;
+        if (SUTH && F.g_inf < 0) bad = true;
+        winf[0] = r.v;
+        winf[1] = (u.v & ~1ll) | (bad ? 1 : 0);
+        winf[2] = v.v;
+        winf[3] = p.v;
+        winf[4] = T.v;
+        winf[5] = F.g_inf;
+    }
+    __syncthreads();
+    for (int idx = tid; idx < EW * EH; idx += NT) {
+        const int lx = idx % EW, ly = idx / EW;
+        int gi = i0 + lx - 2, gj = j0 + ly - 2;
+        bool mirror, inf;
+        curv_source(C, gi, gj, mirror, inf);
+        long long w[6];
+        if (inf) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) w[k] = winf[k];
+        } else {
+            const size_t c = (size_t)gj * nx + gi;
+            const double q0 = load_value(io, cf, cff, c), q1 = load_value(io, cf, cff, nc + c);
+            const double q2 = load_value(io, cf, cff, 2 * nc + c), q3 = load_value(io, cf, cff, 3 * nc + c);
+            fixed_prim<VISC, SUTH>(q0, q1, q2, q3, eR, eU, F, w);
+        }
+        if (mirror) {
+            w[1] = -(w[1] & ~1ll) | (w[1] & 1);
+            w[2] = -w[2];
+        }
+        tl.r[ly][lx] = w[0];
+        tl.u[ly][lx] = w[1];
+        tl.v[ly][lx] = w[2];
+        tl.p[ly][lx] = w[3];
+        if (VISC) tl.T[ly][lx] = w[4];
+        if (SUTH) tl.g[ly][lx] = w[5];
+    }
+    __syncthreads();
+
+    for (int bt = tid >> 5; bt < (NF + 31) / 32; bt += NT / 32) {
+        const int f = bt * 32 + (tid & 31);
+        const bool yd = f >= NFX_;
+        const int g = yd ? f - NFX_ : f;
+        const int fx_ = yd ? g % TX : g % (TX + 1), fy = yd ? g / TX : g / (TX + 1);
+        const int gi = i0 + fx_, gj = j0 + fy;
+        bool bad = false;
+        if (f < NF && (yd ? (gi < nx && gj <= ny) : (gi <= nx && gj < ny))) {
+            const longlong2 *mp = reinterpret_cast<const longlong2 *>(yd ? G.fj + ((size_t)gj * nx + gi)
+                                                                         : G.fi + ((size_t)gj * (nx + 1) + gi));
+            const longlong2 mn = __ldg(mp), ml = __ldg(mp + 3);   // normal; half length, exponent
+            const Fx<0> mnx = {mn.x}, mny = {mn.y};
+            const int ip = (fy + 2) * EW + fx_ + 2;
+            const int sn = yd ? EW : 1, im = ip - sn;
+            const int st = yd ? -1 : EW;   // step along the face: +1 row on i-faces, -1 column on j-faces
+            const long long *pr = &tl.r[0][0], *pu = &tl.u[0][0], *pv = &tl.v[0][0], *pp = &tl.p[0][0];
+            FixedState L, R;
+            Fx<0> uL, uR, vL, vR;
+            fixed_muscl(pr[im - sn], pr[im], pr[ip], pr[ip + sn], F, L.r.v, R.r.v);
+            fixed_muscl_p(pp[im - sn], pp[im], pp[ip], pp[ip + sn], F, L.p, R.p);
+            const long long um = pu[im], up = pu[ip], um2 = pu[im - sn], up2 = pu[ip + sn];
+            const long long vm = pv[im], vp = pv[ip];
+            fixed_muscl(um2, um, up, up2, F, uL.v, uR.v);
+            fixed_muscl(pv[im - sn], vm, vp, pv[ip + sn], F, vL.v, vR.v);
+            unsigned flag = (unsigned)(um | up | um2 | up2);
+            if (outside<1>(uL) || outside<1>(uR) || outside<1>(vL) || outside<1>(vR)) bad = true;
+            L.n = mul<0>(uL, mnx) + mul<0>(vL, mny);
+            R.n = mul<0>(uR, mnx) + mul<0>(vR, mny);
+            L.t = mul<0>(vL, mnx) - mul<0>(uL, mny);
+            R.t = mul<0>(vR, mnx) - mul<0>(uR, mny);
+            Fx<0> v1{0}, v2{0}, ve{0};
+            if (VISC) {
+                const long long *pT = &tl.T[0][0];
+                const longlong2 ca = __ldg(mp + 1), cb = __ldg(mp + 2);
+                const Fx<0> c0 = {ca.x}, c1 = {ca.y}, c2 = {cb.x}, c3 = {cb.y};
+                const long long a0 = pu[im + st], a1 = pu[ip + st], b0 = pu[im - st], b1 = pu[ip - st];
+                flag |= (unsigned)(a0 | a1 | b0 | b1);
+                Fx<0> dVu = {(a0 + a1) - (b0 + b1)};
+                Fx<0> dVv = {(pv[im + st] + pv[ip + st]) - (pv[im - st] + pv[ip - st])};
+                Fx<0> dVT = {(pT[im + st] + pT[ip + st]) - (pT[im - st] + pT[ip - st])};
+                Fx<0> dCu = {up - um}, dCv = {vp - vm}, dCT = {pT[ip] - pT[im]};
+                if (outside<1>(dVu) || outside<1>(dVv) || outside<1>(dVT)) bad = true;
+                // the terms are those of the mantissas times 2^-sh.  On thin cells
+                // (sh < 0) the differences are scaled up first, as far as they allow
+                // (by l1), the terms by the rest: the products then drop no bits that matter
+                const int sh = eR + eU - C.fxv.e - (int)ml.y;
+                int l1 = 0, l2 = 0;
+                if (sh < 0) {
+                    const Fx<0> *d[6] = {&dCu, &dCv, &dCT, &dVu, &dVv, &dVT};
+                    int m = 0;
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) m |= hi_word(d[k]->v) ^ (hi_word(d[k]->v) >> 31);
+                    l1 = min(max(__clz(m) - 3, 0), -sh);
+                    l2 = min(-sh - l1, 30);
+                    if (-sh - l1 > 30) bad = true;
+                    dCu.v <<= l1;
+                    dCv.v <<= l1;
+                    dCT.v <<= l1;
+                    dVu.v <<= l1;
+                    dVv.v <<= l1;
+                    dVT.v <<= l1;
+                }
+                // coefficients below 1/2, across-differences below 1, along-differences below 1/2: gradients below 3/4
+                const Fx<0> ux = mul<0>(dCu, c0) + mul<0>(dVu, c1), uy = mul<0>(dCu, c2) + mul<0>(dVu, c3);
+                const Fx<0> vx = mul<0>(dCv, c0) + mul<0>(dVv, c1), vy = mul<0>(dCv, c2) + mul<0>(dVv, c3);
+                const Fx<0> Tx = mul<0>(dCT, c0) + mul<0>(dVT, c1), Ty = mul<0>(dCT, c2) + mul<0>(dVT, c3);
+                const Fx<0> sxy = half_of(uy + vx);
+                const Fx<0> k0 = {C.fxv.k[0][0]}, k1 = {C.fxv.k[0][1]}, k2 = {C.fxv.k[0][2]}, k3 = {C.fxv.k[0][3]};
+                Fx<0> txx = mul<0>(ux, k0) + mul<0>(vy, k1), tyy = mul<0>(vy, k0) + mul<0>(ux, k1);
+                const Fx<0> txh = mul<0>(sxy, k2);   // half of txy
+                Fx<0> txy = txh + txh;
+                Fx<0> q = mul<0>(mul<0>(Tx, mnx) + mul<0>(Ty, mny), k3);
+                Fx<0> t1 = mul<0>(txx, mnx) + mul<0>(txy, mny), t2 = mul<0>(txy, mnx) + mul<0>(tyy, mny);
+                if (outside<1>(t1) || outside<1>(t2) || outside<1>(q)) bad = true;
+                if (SUTH) {
+                    const long long *pg = &tl.g[0][0];
+                    const Fx<2> mus = {pg[im] + pg[ip]};   // below 4
+                    const Fx<2> a = mul<2>(t1, mus), b = mul<2>(t2, mus), c = mul<2>(q, mus);
+                    if (outside<3>(a) || outside<3>(b) || outside<3>(c)) bad = true;
+                    t1 = to<0>(a);
+                    t2 = to<0>(b);
+                    q = to<0>(c);
+                }
+                const Fx<0> w = half_of(mul<0>(Fx<0>{um + up}, t1) + mul<0>(Fx<0>{vm + vp}, t2)) + q;
+                if (sh < 0) {
+                    v1 = scale_up(t1, l2, bad);
+                    v2 = scale_up(t2, l2, bad);
+                    ve = scale_up(w, l2, bad);
+                } else {
+                    const int r = min(sh, 63);
+                    v1 = {t1.v >> r};
+                    v2 = {t2.v >> r};
+                    ve = {w.v >> r};
+                }
+            }
+            if (flag & 1) bad = true;
+            Fx<0> g4[4];
+            fixed_roe<false>(L, R, F, Fx<0>{0}, Fx<0>{0}, ve, g4, bad);
+            // rotate halves of the momentum fluxes, tested below 1/2
+            const Fx<0> gn = half_of(g4[1]), gt = half_of(g4[2]);
+            if (outside<1>(gn) || outside<1>(gt)) bad = true;
+            const Fx<0> m1 = mul<0>(gn, mnx) - mul<0>(gt, mny), m2 = mul<0>(gn, mny) + mul<0>(gt, mnx);
+            if (!bad) {
+                const double len = __longlong_as_double(ml.x);
+                double *out = yd ? &fc.fy[0][fy][fx_] : &fc.fx[0][fy][fx_];
+                const int ks = yd ? (TY + 1) * TX : TY * (TX + 1);
+                out[0] = (double)g4[0].v * len;
+                out[ks] = (double)(m1.v + m1.v - v1.v) * len;
+                out[2 * ks] = (double)(m2.v + m2.v - v2.v) * len;
+                out[3 * ks] = (double)g4[3].v * len;
+            }
+        }
+        const unsigned left = __ballot_sync(0xffffffffu, bad);
+        if ((tid & 31) == 0) {
+            slow[bt] = left;
+            if (left) fs.any_slow = 1;
+        }
+    }
+    __syncthreads();
+    if (fs.any_slow) {
+        slow_curv_faces<VISC, SUTH, SH>(C, G, io, i0, j0, smem_raw, fc, fs, slow);
+        __syncthreads();
+    }
+
+    for (int cell = tid; cell < TX * TY; cell += NT) {
+        const int tx = cell % TX, ty = cell / TX;
+        const int gi = i0 + tx, gj = j0 + ty;
+        if (gi < nx && gj < ny) {
+            const size_t c = (size_t)gj * nx + gi;
+            const double iv = G.inv_vol[c];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double dX = fc.fx[k][ty][tx + 1] - fc.fx[k][ty][tx];
+                const double dY = fc.fy[k][ty + 1][tx] - fc.fy[k][ty][tx];
+                epilogue_store(io, s1, s2, k * nc + c, -((dX + dY) * (iv * fs.bx[k])));
+            }
+        }
+    }
 }

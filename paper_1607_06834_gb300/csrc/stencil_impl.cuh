@@ -1277,17 +1277,56 @@ static cudaError_t launch_fixed_tiles(const StencilConsts &c, const StencilIO &i
     return cudaGetLastError();
 }
 
+__global__ void __launch_bounds__(256)
+    fixed_metrics_kernel(const double *nx, const double *ny, const double *len, const double *c0, const double *c1,
+                         const double *c2, const double *c3, size_t n, FixedMetric *out)
+{
+    const size_t f = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (f < n) out[f] = fixed_metric(nx[f], ny[f], len[f], c0[f], c1[f], c2[f], c3[f]);
+}
+
+cudaError_t launch_fixed_metrics(const double *nx, const double *ny, const double *len, const double *c0,
+                                 const double *c1, const double *c2, const double *c3, size_t n, FixedMetric *out,
+                                 cudaStream_t s)
+{
+    fixed_metrics_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nx, ny, len, c0, c1, c2, c3, n, out);
+    return cudaGetLastError();
+}
+
+// Curvilinear faces take the small tile at every size: its one round of eight
+// face batches runs the long face code once per CTA (the larger tiles' warps
+// drift apart in it and miss the instruction cache).  FD-JVP with Sutherland's
+// law, us, 16 x 7 / 16 x 16 / 32 x 15: 256 x 128 14.9 / 21.1 / 37.6; 512 x 256
+// 45.0 / 52.5 / 50.8; 1024 x 512 177 / 178 / 182.
+template <bool V, bool SU>
+static cudaError_t launch_fixed_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
+{
+    typedef FixedShapeS SH;
+    const size_t smem = FixedSmem<SU, SH>::bytes;
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(fixed_curv_kernel<V, SU, SH, kFixedMinB>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    dim3 grid((c.nx + SH::TX - 1) / SH::TX, (c.ny + SH::TY - 1) / SH::TY);
+    fixed_curv_kernel<V, SU, SH, kFixedMinB><<<grid, SH::NT, smem, s>>>(c, g, io);
+    return cudaGetLastError();
+}
+
 // The tile by the grid's size (the bits do not depend on it).  FD-JVP, viscous,
-// us a launch, 16 x 7 / 16 x 16 / 32 x 15: 128^2 10.3 / 16.4 / 24.6 (the
-// grid is below one CTA per SM: the smallest chain of rounds wins); 512^2
-// 63.5 / 59.7 / 60.8; 1024^2 264 / 224 / 205 (32 x 15 loads 1.43 cells a cell
-// where 16 x 16 loads 1.56, but needs three full waves of 3 CTAs per SM).
+// us a launch (graph nodes), 16 x 7 / 16 x 16 / 32 x 15: 128^2 8.8 / 15.3 / 23.9
+// (below one CTA per SM the smallest chain of rounds wins); 256^2 20.3 / 21.3 /
+// 24.2; 384^2 37.9 / 37.1 / 44.5; 512^2 63.2 / 59.9 / 59.6; 768^2 138 / 131 /
+// 122; 1024^2 267 / 231 / 212 (32 x 15 loads 1.43 cells a cell where 16 x 16
+// loads 1.56 and 16 x 7 1.96, but wants three waves of 3 CTAs per SM).
 template <bool V, bool SU>
 static cudaError_t launch_fixed_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
     auto tiles = [&](int tx, int ty) { return (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty); };
-    if (tiles(32, 15) >= 3 * 3 * 152) return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
-    if (tiles(16, 16) > 152) return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
+    if (tiles(32, 15) >= 1140) return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
+    if (tiles(16, 16) > 456) return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
     return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
 }
 #endif
@@ -1384,6 +1423,12 @@ cudaError_t launch_cart_batch(const StencilConsts &c, const StencilIO &io, const
 cudaError_t launch_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
 {
     const bool dual = io.dir || io.dirf;
+#ifdef ROK_STENCIL_FAST
+    if (!dual && c.fx.ok && g.fi) {
+        if (!c.viscous) return launch_fixed_curv<false, false>(c, g, io, s);
+        return c.sutherland ? launch_fixed_curv<true, true>(c, g, io, s) : launch_fixed_curv<true, false>(c, g, io, s);
+    }
+#endif
     if (!c.viscous)
         return dual ? launch_curv_t<false, false, Dual>(c, g, io, s) : launch_curv_t<false, false, double>(c, g, io, s);
     if (c.sutherland)
