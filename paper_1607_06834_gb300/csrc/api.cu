@@ -331,6 +331,10 @@ rok_status arnoldi_columns(rok_ctx *c, const double *y, int M)
         }
         if (e != cudaErrorNotSupported || c->fp32) return ROK_ERR_CUDA;
         (void)cudaGetLastError();
+        if (c->ops->gs_column) {
+            CU(c->ops->gs_column(c->w, c->V, N, N, j, j + 1 < M ? 1 : 0, c->pM, st, &c->launches, s));
+            continue;
+        }
         // <v_1, w> and ||w||^2
         CU(c->ops->dot2(c->V, c->w, c->w, c->w, N, c->pA, P, &st->active, s));
         c->launches++;
@@ -807,19 +811,23 @@ static rok_status gmres_solve(rok_ctx *c, const double *y, const double *F0, dou
             } else {
                 if (e != cudaErrorNotSupported) return ROK_ERR_CUDA;
                 (void)cudaGetLastError();
-                CU(c->ops->dot2(c->V, wv, wv, wv, N, c->pA, P, &st->active, s));
-                double *pin = c->pA, *pout = c->pB;
-                for (int q = 1; q <= j + 1; ++q) {
-                    const double *vnext = q <= j ? c->V + (size_t)q * N : nullptr;
-                    CU(c->ops->mgs(wv, c->V + (size_t)(q - 1) * N, vnext, N, pin, P,
-                                   &st->H[(q - 1) * kMaxKrylov + j], pout, q == 1, st, s));
-                    double *t = pin;
-                    pin = pout;
-                    pout = t;
+                if (c->ops->gs_column) {
+                    CU(c->ops->gs_column(wv, c->V, N, N, j, 1, c->pM, st, &c->launches, s));
+                } else {
+                    CU(c->ops->dot2(c->V, wv, wv, wv, N, c->pA, P, &st->active, s));
+                    double *pin = c->pA, *pout = c->pB;
+                    for (int q = 1; q <= j + 1; ++q) {
+                        const double *vnext = q <= j ? c->V + (size_t)q * N : nullptr;
+                        CU(c->ops->mgs(wv, c->V + (size_t)(q - 1) * N, vnext, N, pin, P,
+                                       &st->H[(q - 1) * kMaxKrylov + j], pout, q == 1, st, s));
+                        double *t = pin;
+                        pin = pout;
+                        pout = t;
+                    }
+                    CU(c->ops->normalize(wv, c->V + (size_t)(j + 1) * N, N, pin, P,
+                                         &st->H[(j + 1) * kMaxKrylov + j], j + 1, st, s));
+                    c->launches += 3 + j;
                 }
-                CU(c->ops->normalize(wv, c->V + (size_t)(j + 1) * N, N, pin, P,
-                                     &st->H[(j + 1) * kMaxKrylov + j], j + 1, st, s));
-                c->launches += 3 + j;
             }
             CU(c->ops->gmres_givens(j, st, s));
             c->launches++;

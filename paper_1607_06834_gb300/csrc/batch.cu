@@ -211,6 +211,20 @@ rok_status enqueue_step(rok_batch *b, double *y, int M)
             io.s1_dev = &b->st[0].inv_eps;
             io.active = &b->st[0].active;
             if ((r = stencil(b, io)) != ROK_OK) return r;
+            if (o.gs_pass) {   // FMA build: four basis vectors a pass
+                const int blocks = (j + 4) / 4;
+                auto in_block = [&](int q) { return j + 1 - 4 * q < 4 ? j + 1 - 4 * q : 4; };
+                for (int q = -1; q < blocks; ++q) {
+                    CU(o.gs_pass(b->w, b->V, ldv, j, q < 0 ? 0 : q, q < 0 ? 0 : in_block(q), q + 1,
+                                 q + 1 < blocks ? in_block(q + 1) : 0, j + 1 < M ? 1 : 0, b->pM, sg, b->cpc, s));
+                    b->launches++;
+                }
+                if (j + 1 < M) {
+                    CU(o.gs_normalize(b->w, b->V, ldv, j, sg, b->vcpc, s));
+                    b->launches++;
+                }
+                continue;
+            }
             CU(o.dot2(b->V, b->w, b->w, b->w, b->pA, sg, 1, b->cpc, s));
             b->launches++;
             double *pin = b->pA, *pout = b->pB;
@@ -403,7 +417,7 @@ rok_status rok_batch_init(rok_batch **out, const rok_problem_desc *descs, int co
               cudaMalloc(&b->st, count * sizeof(StepState)) == cudaSuccess &&
               al(&b->V, (size_t)(b->mmax + 1) * N) && al(&b->w, N) && al(&b->t0, N) &&
               al(&b->pA, 2 * (size_t)b->nchunks) && al(&b->pB, 2 * (size_t)b->nchunks) &&
-              al(&b->pM, (size_t)(b->mmax > 0 ? b->mmax : 1) * b->nchunks) && al(&b->d_h, count) &&
+              al(&b->pM, (size_t)(b->mmax > 8 ? b->mmax : 8) * b->nchunks) && al(&b->d_h, count) &&
               cudaMallocHost(&b->h_st, count * sizeof(StepState)) == cudaSuccess;
     for (int i = 0; i < 4 && ok; ++i) ok = al(&b->F[i], N) && al(&b->K[i], N);
     if (!ok) { free_batch(b); return ROK_ERR_NOMEM; }
@@ -550,8 +564,12 @@ rok_status rok_batch_tune(rok_batch *b, const double *y, rok_batch_tuning *out)
         const int c = kCpcCandidates[q];
         float ms = 0.0f;
         r = time_ms(b, 3, [&] {
-            return b->bops->mgs(b->t0, b->V, b->total, 1, 0, b->pA, b->pB, sg, c, b->stream) == cudaSuccess
-                       ? ROK_OK : ROK_ERR_CUDA; }, &ms);
+            // FMA build: a full block of the basis, projected on again
+            const int nv = b->mmax + 1 < 4 ? b->mmax + 1 : 4;
+            const cudaError_t e =
+                b->bops->gs_pass ? b->bops->gs_pass(b->t0, b->V, b->total, kMaxKrylov - 1, 0, nv, 0, nv, 0, b->pM, sg, c, b->stream)
+                                 : b->bops->mgs(b->t0, b->V, b->total, 1, 0, b->pA, b->pB, sg, c, b->stream);
+            return e == cudaSuccess ? ROK_OK : ROK_ERR_CUDA; }, &ms);
         if (r != ROK_OK) return r;
         t.mgs_ms[q] = ms;
         if (best_m < 0.0f || ms < best_m) { best_m = ms; t.chunks_per_cta = c; }

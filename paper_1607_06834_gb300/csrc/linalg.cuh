@@ -54,6 +54,12 @@ struct StepState {
     double gcoef[kMaxKrylov + 1];  // coefficients of the GMRES update x += V gcoef
     GmresState gm;
     double gram[kMaxKrylov];       // <v_{i+1}, v_i> of the basis (FMA-build two-vector passes)
+    // FMA-build block passes (gs_column): <v_i, v_k> with the earlier vectors k of
+    // i's block of four, the block's coefficients, sum of the column's squared
+    // coefficients, 1 / h_{j+1,j}, and the arrivals of the running launch (0 at rest)
+    double bgram[kMaxKrylov][3];
+    double gs_h[4], gs_ssq, gs_rh;
+    unsigned gs_count;
 };
 
 // ---- rounding-mode dependent vector kernels (linalg_impl.cuh, compiled twice) ----
@@ -108,6 +114,12 @@ struct LinalgOps {
     cudaError_t (*arnoldi_column)(const double *w, void *V, int fp32, size_t ldv, size_t n, int j, int next, int P,
                                   double *partA, double *partB, unsigned *cnt, StepState *st, int ctas,
                                   cudaStream_t s);
+    // One whole Arnoldi column j by block passes, a few launches (FMA build; null
+    // in the strict build, which takes dot2 + mgs + normalize): as arnoldi_column
+    // for a binary64 basis of any length.  w is updated in place, part holds 8 P
+    // partials, *launches is increased by the kernels launched.
+    cudaError_t (*gs_column)(double *w, double *V, size_t ldv, size_t n, int j, int next, double *part, StepState *st,
+                             long long *launches, cudaStream_t s);
     // co-resident CTAs of arnoldi_column on this device (0 if cooperative launch is unavailable)
     int (*arnoldi_column_ctas)(int sms);
     // v_1 = (T)F1 / ||(T)F1|| (T = binary64 or binary32); beta = 0: empty basis
@@ -151,7 +163,16 @@ struct BatchOps {
     cudaError_t (*eps)(const double *part, const BSeg &sg, int ninst, cudaStream_t s);
     cudaError_t (*first_normalize)(const double *F, double *V0, const double *part, const BSeg &sg, int cpc,
                                    cudaStream_t s);
-    // MGS pass i (1 <= i <= j + 1) of column j
+    // One block pass of column j (FMA build; null in the strict build): w -= the
+    // previous block's nb projections (block b of four vectors, coefficients in the
+    // step states), then the products of w with the nn vectors of block b2, or
+    // ||w||^2 when nn = 0 (then, with next, h_{j+1,j}, the breakdown test and
+    // its reciprocal).  part: 8 nchunks partials.
+    cudaError_t (*gs_pass)(double *w, const double *V, size_t ldv, int j, int b, int nb, int b2, int nn, int next,
+                           double *part, const BSeg &sg, int cpc, cudaStream_t s);
+    // v_{j+1} = w / h_{j+1,j} (FMA build)
+    cudaError_t (*gs_normalize)(const double *w, double *V, size_t ldv, int j, const BSeg &sg, int cpc, cudaStream_t s);
+    // MGS pass i (1 <= i <= j + 1) of column j (strict build; null in the FMA build, as normalize)
     cudaError_t (*mgs)(double *w, const double *V, size_t ldv, int i, int j, const double *pin, double *pout,
                        const BSeg &sg, int cpc, cudaStream_t s);
     cudaError_t (*normalize)(const double *w, double *V, size_t ldv, int column, const double *pin, const BSeg &sg,
