@@ -1323,11 +1323,27 @@ __device__ __forceinline__ Quad ld_quad(const double *p)
     asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(q.x), "=d"(q.y), "=d"(q.z), "=d"(q.w) : "l"(p));
     return q;
 }
+// binary32 to binary64 on the integer pipe: the conversion instruction runs at
+// the FP64 rate (2 lanes per SM and clock) and cost as much as the product it
+// feeds.  A normal number's exponent is rebiased by 896 and its fraction moved up
+// by 29 bits; zeros keep their sign; subnormals, infinities and NaN take the
+// instruction (out of line: a predicated conversion would be issued for all).
+// 512^2, 20 vectors: projections 97 -> 66 us, stage vectors 83 -> 43 us a launch.
+__device__ __noinline__ double widen_special(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    const unsigned m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return widen_special(x);
+    const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
 // four consecutive binary32 basis values (one 16-byte load), exactly as binary64
 __device__ __forceinline__ Quad ld_quad(const float *p)
 {
     const float4 f = __ldg(reinterpret_cast<const float4 *>(p));
-    return Quad{(double)f.x, (double)f.y, (double)f.z, (double)f.w};
+    return Quad{widen(f.x), widen(f.y), widen(f.z), widen(f.w)};
 }
 
 template <int E, class T>
