@@ -323,7 +323,7 @@ rok_status arnoldi_columns(rok_ctx *c, const double *y, int M)
         cudaError_t e = cudaErrorNotSupported;
         if (c->col_ctas > 0 && c->persistent)
             e = c->ops->arnoldi_column(c->w, Vb, c->fp32 ? 1 : 0, N, N, j, j + 1 < M ? 1 : 0, P,
-                                       c->fp32 ? c->pM : c->pA, c->pB,
+                                       c->fp32 || c->ops->gs_column ? c->pM : c->pA, c->pB,
                                        c->colcnt + column_counter_offset(j), st, c->col_ctas, s);
         if (e == cudaSuccess) {
             c->launches++;
@@ -395,8 +395,8 @@ rok_status enqueue_rok_body(rok_ctx *c, double *y, int M)
             if ((r = stencil(c, io)) != ROK_OK) return r;
         }
         if (M > 0) {
-            CU(c->ops->multidot(c->F[i], Vb, c->fp32 ? 1 : 0, N, N, c->pM, P, st, s));
-            CU(c->ops->stage_solve(i, kRokGammaOff[i], c->pM, P, st, s));
+            CU(c->ops->multidot(c->F[i], Vb, c->fp32 ? 1 : 0, N, N, c->pM, c->Pm, st, s));
+            CU(c->ops->stage_solve(i, kRokGammaOff[i], c->pM, c->Pm, st, s));
             c->launches += 2;
         }
         CU(c->ops->stage_vec(c->K[i], c->F[i], Vb, c->fp32 ? 1 : 0, N, N, i, st, c->egrid, s));
@@ -502,6 +502,11 @@ rok_status rok_init(rok_ctx **out, const rok_problem_desc *d, void *stream)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     c->P = reduction_blocks(c->N);
+    c->Pm = c->P;
+    if (!c->strict) {   // the FMA build splits short vectors finer than the 2048-entry chunks
+        const size_t fine = (c->N + 511) / 512;
+        c->Pm = std::max(c->P, (int)std::min<size_t>(fine, 256));
+    }
     c->egrid = 8 * sms;
     c->ops = c->strict ? &strict::ops : &fast::ops;
 
@@ -538,7 +543,7 @@ rok_status rok_init(rok_ctx **out, const rok_problem_desc *d, void *stream)
     auto al = [&](double **p, size_t n) { return cudaMalloc(p, n * sizeof(double)) == cudaSuccess; };
     bool ok = al(&c->V, (size_t)(c->mmax + 1) * N) && al(&c->w, N) && al(&c->t0, N) && al(&c->t1, N) &&
               al(&c->t2, N) && al(&c->pA, 4 * (size_t)c->P) && al(&c->pB, 2 * (size_t)c->P) &&
-              al(&c->pM, (size_t)(kMaxKrylov + 2) * c->P);
+              al(&c->pM, (size_t)(kMaxKrylov + 2) * c->Pm);
     for (int i = 0; i < 4 && ok; ++i) ok = al(&c->F[i], N) && al(&c->K[i], N);
     if (ok && c->fp32) ok = cudaMalloc(&c->Vf, (size_t)(c->mmax + 1) * N * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->st, sizeof(StepState)) == cudaSuccess;
@@ -804,7 +809,7 @@ static rok_status gmres_solve(rok_ctx *c, const double *y, const double *F0, dou
             if ((r = apply_op(c->V + (size_t)j * N, wv, &st->active)) != ROK_OK) return r;
             cudaError_t e = cudaErrorNotSupported;
             if (persistent)
-                e = c->ops->arnoldi_column(wv, c->V, 0, N, N, j, 1, P, c->pA, c->pB,
+                e = c->ops->arnoldi_column(wv, c->V, 0, N, N, j, 1, P, c->ops->gs_column ? c->pM : c->pA, c->pB,
                                            c->colcnt + column_counter_offset(j), st, c->col_ctas, s);
             if (e == cudaSuccess) {
                 c->launches++;

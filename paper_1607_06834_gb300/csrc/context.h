@@ -23,6 +23,7 @@ struct rok_ctx {
     int kind = 0;
     size_t nc = 0, N = 0;
     int P = 0;                 // CTAs (partials) of a reduction over N entries
+    int Pm = 0;                // partials a value in pM (at least P)
     int egrid = 0;             // CTAs of the element-wise kernels
     const LinalgOps *ops = nullptr;
     int mmax = 0;

@@ -74,7 +74,8 @@ struct LinalgOps {
     // hn = sqrt(tree(pin)); breakdown / beta tests; v = w * (1/hn); *hsub = hn (nullable)
     cudaError_t (*normalize)(const double *w, double *v, size_t n, const double *pin, int P, double *hsub,
                              int column, StepState *st, cudaStream_t s);
-    // pout[m*P + b] = <V_m, F> over CTA b's entries, m < meff; V binary64 or (fp32) binary32
+    // pout[m*P + b] = <V_m, F> over CTA b's entries, m < meff; V binary64 or (fp32) binary32;
+    // P >= reduction_blocks(n) (the FMA build takes up to P CTAs)
     cudaError_t (*multidot)(const double *F, const void *V, int fp32, size_t ldv, size_t n, double *pout, int P,
                             const StepState *st, cudaStream_t s);
     // stage i: phi, rhs = h phi + h H sum_j gam_ij lam_j, lam_i by LU, cvec_i = lam_i - h phi
@@ -99,7 +100,8 @@ struct LinalgOps {
     // co-resident): h_ij = <v_i, w>, w -= h_ij v_i for i = 0..j (modified
     // Gram-Schmidt), then, when next != 0, h_{j+1,j} = ||w||, the breakdown test
     // and v_{j+1} = w * (1/h_{j+1,j}).  w and the next basis vector stay in
-    // registers between passes; partA holds 4P partials, partB 2P; cnt[0 ..
+    // registers between passes; partA holds 4P partials, partB 2P (FMA build,
+    // binary64 basis: partA max(4P, 6 ceil(n / 512)), partB unused); cnt[0 ..
     // j + 2) are the arrival counters of the partial generations, zero on entry
     // (column_counter_offset).  Strict build: the same arithmetic as dot2 + mgs
     // + normalize.  FMA build: two basis vectors a pass (MGS to rounding); the

@@ -1362,10 +1362,13 @@ __global__ void __launch_bounds__(kEvenThreads, 1)
     const size_t nq = (hi - lo) / 4;   // quads of this CTA (L, n multiples of 4)
     const int kv = threadIdx.x < nq ? (int)((nq - threadIdx.x + TH - 1) / TH) : 0;
     const double *F4 = F + lo + 4 * (size_t)threadIdx.x;
+    if ((threadIdx.x & ~31u) >= nq) {   // a warp without entries: its share is zero (see pair_kernel)
+        for (int i = threadIdx.x & 31; i < m; i += 32) ws[i][threadIdx.x >> 5] = 0.0;
+    }
     Quad f[E4];
 #pragma unroll
     for (int k = 0; k < E4; ++k) f[k] = k < kv ? ld_quad(F4 + (size_t)4 * k * TH) : Quad{0.0, 0.0, 0.0, 0.0};
-    for (int g = 0; g < m; g += 16) {
+    for (int g = 0; g < m && (threadIdx.x & ~31u) < nq; g += 16) {
         const int cnt = m - g < 16 ? m - g : 16;   // uniform
         double t[16];
 #pragma unroll
@@ -1701,6 +1704,38 @@ __global__ void __launch_bounds__(RT) first_normalize_kernel(const double *__res
     store8(V0, e0, n, x);
 }
 
+#ifdef ROK_LINALG_FAST
+// The instantiation of arnoldi_pair_kernel for e entries a thread: the smallest
+// that holds them.  An FP64 instruction whose lanes are all predicated off still
+// occupies the unit, so a loose fit costs as much as the entries it could hold
+// (64 x 64 cells, 4 entries of 8: 6.8 us a pass, as 7 of 8 on 256 x 512).
+struct PairKernel {
+    int E;
+    const void *fn;
+    size_t smem;
+};
+template <int E>
+PairKernel pair_kernel_of()
+{
+    return {E, (const void *)arnoldi_pair_kernel<E>, pair_stage_bytes<E>()};
+}
+static PairKernel pair_kernel(int e)
+{
+    if (e <= 1) return pair_kernel_of<1>();
+    if (e <= 2) return pair_kernel_of<2>();
+    if (e <= 3) return pair_kernel_of<3>();
+    if (e <= 4) return pair_kernel_of<4>();
+    if (e <= 5) return pair_kernel_of<5>();
+    if (e <= 6) return pair_kernel_of<6>();
+    if (e <= 7) return pair_kernel_of<7>();
+    if (e <= 8) return pair_kernel_of<8>();
+    if (e <= 10) return pair_kernel_of<10>();
+    if (e <= 12) return pair_kernel_of<12>();
+    if (e <= 14) return pair_kernel_of<14>();
+    return pair_kernel_of<16>();
+}
+#endif
+
 static int arnoldi_column_ctas(int sms)
 {
     int dev = 0, coop = 0, p64 = 0, p32 = 0;
@@ -1717,13 +1752,11 @@ static int arnoldi_column_ctas(int sms)
     // the binary64 column runs as arnoldi_pair_kernel, kEvenThreads threads a CTA
     // and a dynamic staging buffer: its grid is ctas RT / kEvenThreads, which must
     // be co-resident too
-    const void *pk[3] = {(const void *)arnoldi_pair_kernel<8>, (const void *)arnoldi_pair_kernel<14>,
-                         (const void *)arnoldi_pair_kernel<16>};
-    const size_t pb[3] = {pair_stage_bytes<8>(), pair_stage_bytes<14>(), pair_stage_bytes<16>()};
-    for (int i = 0; i < 3; ++i) {
-        if (cudaFuncSetAttribute(pk[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pb[i]) != cudaSuccess)
-            return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pe, pk[i], kEvenThreads, pb[i]) != cudaSuccess) return 0;
+    for (int E = 1; E <= kEvenPerThread; ++E) {
+        const PairKernel k = pair_kernel(E);
+        if (k.E != E) continue;
+        if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess) return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pe, k.fn, kEvenThreads, k.smem) != cudaSuccess) return 0;
         if (pe * kEvenThreads < p64 * RT) p64 = pe * kEvenThreads / RT;
     }
 #endif
@@ -1755,29 +1788,26 @@ static cudaError_t arnoldi_column(const double *w, void *V, int fp32, size_t ldv
     double *Vd = static_cast<double *>(V);
     double tol = 1e-12;
 #ifdef ROK_LINALG_FAST
-    // even split: Ge CTAs of kEvenThreads threads and L entries each
-    const int Gmax = ctas * RT / kEvenThreads;
-    const int Ge = P < Gmax ? P : Gmax;
-    size_t L = (n + Ge - 1) / Ge;
-    L += L & 1;
+    // even split: Ge CTAs of kEvenThreads threads and L entries each; down to one
+    // entry a thread, so that small vectors take many SMs, every CTA with at least
+    // one entry.  16k entries (64 x 64 cells), 12 columns: 8 CTAs of 4 entries a
+    // thread 352 us, 32 of 1 218 us; the projections 18 -> 6 us a launch
+    const int Gmax = min(ctas * RT / kEvenThreads, kEvenMaxGrid);
+    const size_t want = (n + kEvenThreads - 1) / kEvenThreads;
+    int Ge = want < (size_t)Gmax ? (int)want : Gmax;
+    auto range = [&] {
+        const size_t l = (n + Ge - 1) / Ge;
+        return l + (l & 1);
+    };
+    while (Ge > 1 && (size_t)(Ge - 1) * range() >= n) --Ge;
+    size_t L = Ge > 0 ? range() : 0;
     if (Ge < 1 || L > (size_t)kEvenThreads * kEvenPerThread || Ge > kEvenMaxGrid) return cudaErrorNotSupported;
     // the bulk copies of the CTA ranges want 16-byte aligned starts and lengths
     if ((n & 1) || (ldv & 1) || ((uintptr_t)Vd & 15)) return cudaErrorNotSupported;
-    void *eargs[] = {&w, &Vd, &ldv, &n, &j, &next, &L, &partA, &partB, &cnt, &st, &tol};
-    // entries per thread: the smallest instantiation that holds L / kEvenThreads
-    const void *kern;
-    size_t smem;
-    if (L <= (size_t)kEvenThreads * 8) {
-        kern = (const void *)arnoldi_pair_kernel<8>;
-        smem = pair_stage_bytes<8>();
-    } else if (L <= (size_t)kEvenThreads * 14) {
-        kern = (const void *)arnoldi_pair_kernel<14>;
-        smem = pair_stage_bytes<14>();
-    } else {
-        kern = (const void *)arnoldi_pair_kernel<16>;
-        smem = pair_stage_bytes<16>();
-    }
-    return cudaLaunchCooperativeKernel(kern, dim3(Ge), dim3(kEvenThreads), eargs, smem, s);
+    double *partP = partA + 4 * (size_t)Ge;   // partA: the even passes' two sums and the next column's Gram partials
+    void *eargs[] = {&w, &Vd, &ldv, &n, &j, &next, &L, &partA, &partP, &cnt, &st, &tol};
+    const PairKernel k = pair_kernel((int)((L + kEvenThreads - 1) / kEvenThreads));
+    return cudaLaunchCooperativeKernel(k.fn, dim3(Ge), dim3(kEvenThreads), eargs, k.smem, s);
 #else
     void *args[] = {&w, &Vd, &ldv, &n, &j, &next, &P, &partA, &partB, &cnt, &st, &tol};
     return cudaLaunchCooperativeKernel((const void *)arnoldi_column_kernel<double>, dim3(G), dim3(RT), args, 0, s);
@@ -2674,21 +2704,24 @@ static cudaError_t multidot(const double *F, const void *V, int fp32, size_t ldv
                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
                 sms = -1;
         }
-        const int G = sms > 0 && P > sms ? sms : P;
-        size_t L = (n + G - 1) / G;
-        L = (L + 3) & ~(size_t)3;
+        int G = sms > 0 && P > sms ? sms : P;
+        auto range = [&] { return ((n + G - 1) / G + 3) & ~(size_t)3; };
+        while (G > 1 && (size_t)(G - 1) * range() >= n) --G;   // every CTA has entries
+        const size_t L = range();
         // loads of entry quads: lengths multiples of 4, aligned starts
         const uintptr_t va = fp32 ? 15 : 31;
         if (sms > 0 && L <= (size_t)kEvenThreads * kEvenPerThread && !(n & 3) && !(ldv & 3) &&
             !((uintptr_t)F & 31) && !((uintptr_t)V & va)) {
-            const bool e8 = L <= (size_t)kEvenThreads * 8;
+            const bool e4 = L <= (size_t)kEvenThreads * 4, e8 = L <= (size_t)kEvenThreads * 8;
             if (fp32) {
                 const float *Vf = static_cast<const float *>(V);
-                if (e8) multidot_even_kernel<8, float><<<G, kEvenThreads, 0, s>>>(F, Vf, ldv, n, L, pout, P, st);
+                if (e4) multidot_even_kernel<4, float><<<G, kEvenThreads, 0, s>>>(F, Vf, ldv, n, L, pout, P, st);
+                else if (e8) multidot_even_kernel<8, float><<<G, kEvenThreads, 0, s>>>(F, Vf, ldv, n, L, pout, P, st);
                 else multidot_even_kernel<16, float><<<G, kEvenThreads, 0, s>>>(F, Vf, ldv, n, L, pout, P, st);
             } else {
                 const double *Vd = static_cast<const double *>(V);
-                if (e8) multidot_even_kernel<8, double><<<G, kEvenThreads, 0, s>>>(F, Vd, ldv, n, L, pout, P, st);
+                if (e4) multidot_even_kernel<4, double><<<G, kEvenThreads, 0, s>>>(F, Vd, ldv, n, L, pout, P, st);
+                else if (e8) multidot_even_kernel<8, double><<<G, kEvenThreads, 0, s>>>(F, Vd, ldv, n, L, pout, P, st);
                 else multidot_even_kernel<16, double><<<G, kEvenThreads, 0, s>>>(F, Vd, ldv, n, L, pout, P, st);
             }
             return cudaGetLastError();
