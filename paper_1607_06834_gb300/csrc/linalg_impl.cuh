@@ -1222,25 +1222,26 @@ __global__ void __launch_bounds__(kEvenThreads, 1)
     }
     if (!next) return;
     const bool good = pair_wait<1>(cnt + P, G, &st->status, pin, sh4, &ok);
-    // the norm, the breakdown test and the reciprocal by thread 0 (FP64
-    // square roots and divisions in every warp would cost each sub-partition)
+    // the norm, the breakdown test and the reciprocal by thread 0 (in every warp
+    // they would cost each sub-partition): the test on the squares and one reciprocal
+    // square root, a chain of half a dozen FP64 instructions where two square roots
+    // and a division were some sixty (0.5 us a column)
+    double hn2 = 0.0;
     if (threadIdx.x == 0 && good) {
-        const double hn2 = quad_total(sh4, 0);
-        const double hn = sqrt(hn2);
-        const double wnorm0 = sqrt(ssq + hn2);   // ||J v_j||
-        brk = !(hn > brk_tol * wnorm0);
-        sh[0] = 1.0 / hn;
-        if (blockIdx.x == 0) {
-            st->wnorm0 = wnorm0;
-            if (brk) {
-                st->active = 0;
-                st->meff = j + 1;
-            } else {
-                st->H[(j + 1) * kMaxKrylov + j] = hn;
-            }
-        }
+        hn2 = quad_total(sh4, 0);
+        brk = !(hn2 > (brk_tol * brk_tol) * (ssq + hn2));
+        sh[0] = rsqrt(hn2);
     }
     __syncthreads();
+    if (threadIdx.x == 0 && blockIdx.x == 0 && ok) {
+        st->wnorm0 = sqrt(ssq + hn2);   // ||J v_j||
+        if (brk) {
+            st->active = 0;
+            st->meff = j + 1;
+        } else {
+            st->H[(j + 1) * kMaxKrylov + j] = hn2 * sh[0];
+        }
+    }
     if (!ok || brk) return;
     const double r = sh[0];
     // v_{j+1}, and the partials of <v_{j+1}, v_j> (v_j: the last vector used)
