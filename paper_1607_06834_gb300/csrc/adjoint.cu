@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(CT) vjp_cell_kernel(const StencilConsts C, con
     if (t >= nc) return;
     const int i = (int)(t % nx), j = (int)(t / nx);
     auto xf = [&](int fi, int fj) -> size_t { return (size_t)wrapi(fj, ny) * nx + wrapi(fi, nx); };
-    const double a1 = (1.0 + C.c_lo) - C.c_hi;
+    const double a1 = 1.0 + (C.c_lo - C.c_hi);   // one rounding, none at kappa = 1/3: its error is common to all terms
     double Pb[4] = {0.0, 0.0, 0.0, 0.0}, Tb = 0.0;
     // MUSCL: the cell is m2 of face +2, m1 of face +1, p1 of face 0, p2 of face -1
 #pragma unroll
@@ -1212,7 +1212,7 @@ __global__ void __launch_bounds__(CT) curv_vjp_cell_kernel(const StencilConsts C
     auto FY = [&](int q, int a, int b) -> double {
         return (a >= 0 && a < nx && b >= 0 && b <= ny) ? fy[q * nfy + (size_t)b * nx + a] : 0.0;
     };
-    const double a1 = (1.0 + C.c_lo) - C.c_hi;
+    const double a1 = 1.0 + (C.c_lo - C.c_hi);   // one rounding, none at kappa = 1/3: its error is common to all terms
     int ex[3], ey[3];
     bool flx[3], fly[3];
     const int nix = ext_images(i, nx, C.bc[0], C.bc[1], ex, flx);
