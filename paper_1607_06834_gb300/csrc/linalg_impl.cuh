@@ -1440,6 +1440,66 @@ __global__ void __launch_bounds__(kEvenThreads, 1)
             pout[(size_t)(i / (P - (int)gridDim.x)) * P + gridDim.x + i % (P - (int)gridDim.x)] = 0.0;
 }
 
+// The same for longer ranges: the CTA's range in tiles of E entries a thread, the
+// lanes' sums of a group of vectors kept over the tiles and reduced once (the
+// chunked kernel adds a lane tree of 16 FP64 instructions to every 128
+// multiply-adds).  F is read once a group.  1024^2, 20 vectors: 196 -> 161 us a launch
+// (HBM 104, FP64 140).
+template <int E>
+__global__ void __launch_bounds__(kEvenThreads, 1)
+    multidot_long_kernel(const double *__restrict__ F, const double *__restrict__ V, size_t ldv, size_t n, size_t L,
+                         double *__restrict__ pout, int P, const StepState *st)
+{
+    constexpr int TH = kEvenThreads, NW = kEvenThreads / 32, E4 = E / 4;
+    static_assert(NW == 16, "the CTA sum below adds 16 warp sums");
+    __shared__ double ws[kMaxKrylov][NW];
+    const int m = st->meff;
+    const size_t lo = (size_t)blockIdx.x * L;
+    const size_t hi = lo + L < n ? lo + L : n;
+    const size_t nq = (hi - lo) / 4;   // quads of this CTA (L, n multiples of 4)
+    for (int g = 0; g < m; g += 16) {
+        const int cnt = m - g < 16 ? m - g : 16;   // uniform
+        double t[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) t[q] = 0.0;
+        for (size_t q0 = threadIdx.x; q0 < nq; q0 += (size_t)E4 * TH) {
+            Quad f[E4];
+#pragma unroll
+            for (int k = 0; k < E4; ++k)
+                f[k] = q0 + (size_t)k * TH < nq ? ld_quad(F + lo + 4 * (q0 + (size_t)k * TH)) : Quad{0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                if (q < cnt) {
+                    const double *v = V + (size_t)(g + q) * ldv + lo;
+                    double s = t[q];
+#pragma unroll
+                    for (int k = 0; k < E4; ++k)
+                        if (q0 + (size_t)k * TH < nq) {
+                            const Quad x = ld_quad(v + 4 * (q0 + (size_t)k * TH));
+                            s = x.x * f[k].x + s;
+                            s = x.y * f[k].y + s;
+                            s = x.z * f[k].z + s;
+                            s = x.w * f[k].w + s;
+                        }
+                    t[q] = s;
+                }
+        }
+        if (cnt > 8) multidot_group<16>(t, g, m, ws);
+        else if (cnt > 4) multidot_group<8>(t, g, m, ws);
+        else multidot_group<4>(t, g, m, ws);
+    }
+    __syncthreads();
+    if (threadIdx.x < m) {
+        const double *w = ws[threadIdx.x];
+        const double s = (((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]))) +
+                         (((w[8] + w[9]) + (w[10] + w[11])) + ((w[12] + w[13]) + (w[14] + w[15])));
+        pout[(size_t)threadIdx.x * P + blockIdx.x] = s;
+    }
+    if (blockIdx.x == 0)   // the chunk slots past the grid
+        for (int i = threadIdx.x; i < m * (P - (int)gridDim.x); i += TH)
+            pout[(size_t)(i / (P - (int)gridDim.x)) * P + gridDim.x + i % (P - (int)gridDim.x)] = 0.0;
+}
+
 // ---- stage vectors k = sum_i c_i V_i + h F, FMA build: quads of entries ---------
 // Each thread forms four consecutive entries (32-byte loads, four independent
 // FMA chains in the basis order of stage_vec_kernel, so the same values), one
@@ -2775,6 +2835,11 @@ static cudaError_t multidot(const double *F, const void *V, int fp32, size_t ldv
         const size_t L = range();
         // loads of entry quads: lengths multiples of 4, aligned starts
         const uintptr_t va = fp32 ? 15 : 31;
+        if (!fp32 && sms > 0 && L > (size_t)kEvenThreads * kEvenPerThread && !(n & 3) && !(ldv & 3) &&
+            !((uintptr_t)F & 31) && !((uintptr_t)V & 31)) {
+            multidot_long_kernel<8><<<G, kEvenThreads, 0, s>>>(F, static_cast<const double *>(V), ldv, n, L, pout, P, st);
+            return cudaGetLastError();
+        }
         if (sms > 0 && L <= (size_t)kEvenThreads * kEvenPerThread && !(n & 3) && !(ldv & 3) &&
             !((uintptr_t)F & 31) && !((uintptr_t)V & va)) {
             const bool e4 = L <= (size_t)kEvenThreads * 4, e8 = L <= (size_t)kEvenThreads * 8;

@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
 
 # 77220 = 152 * 508 + 4: rounding the range up to a multiple of 4 would leave the last of 152 CTAs empty
 SIZES = [40, 510, 512, 514, 1026, 16384, 20004, 77220, 77824, 79000, 233472, 311300, 400000, 544768, 622592, 700000,
-         900000, 1000000, 1245184]
+         900000, 1000000, 1245184, 1245188, 1300004, 2500000]   # the last three: tiles of a longer range
 
 
 @pytest.mark.parametrize('n', SIZES)
