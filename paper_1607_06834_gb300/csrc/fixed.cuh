@@ -12,8 +12,8 @@
 // Fx<S> holds a number x with |x| < 2^S as the integer x 2^(62 - S).  Scales
 // are compile-time constants; products add them.  Nothing wraps as long as
 // every operand of a product stays below 2^62 in magnitude; callers test the
-// values that the bounds of the inputs do not keep there, and discard a result
-// whose test failed.
+// values that the bounds of the inputs do not keep there (reciprocals by the
+// lower end of in_window), and discard a result whose test failed.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -107,11 +107,14 @@ __device__ __forceinline__ bool outside(Fx<S> a)
     return (unsigned)(hi_word(a.v) + (1 << (30 - LOG))) >= (unsigned)(2 << (30 - LOG));
 }
 
-// x in [2^(S - L), 2^S), on the high word
+// x in [2^(S - L) (1 + 2^(L - 30)), 2^S), on the high word.  The lower end is left
+// out: its reciprocal (or reciprocal root) is a power of two that does not fit the
+// 62 bits, and its high limb would wrap to the negative number.
 template <int L, int S>
 __device__ __forceinline__ bool in_window(Fx<S> a)
 {
-    return (unsigned)(hi_word(a.v) - (1 << (30 - L))) < (unsigned)((1 << 30) - (1 << (30 - L)));
+    constexpr unsigned lo = (1u << (30 - L)) + 1;
+    return (unsigned)hi_word(a.v) - lo < (1u << 30) - lo;
 }
 
 // mul with a test that the result is below 2^(S - LOG) in magnitude, made on
@@ -155,7 +158,7 @@ __device__ __forceinline__ Fx<S> from_double(double x, int e, bool &bad)
 }
 
 // z = 1/sqrt(x) as Fx<L/2> and s = sqrt(x) as Fx<0> for x in [2^-L, 1), L = 6
-// or 8: the hardware's binary32 estimate z0 (relative error about 2^-22) and
+// or 8, the lower end excluded (in_window): the hardware's binary32 estimate z0 (relative error about 2^-22) and
 // one third-order step, with e = 1 - x z0^2: z = z0 (1 + e/2 + 3 e^2/8)
 // (Householder's method), error O(e^3) below the last bit.  z0 has FB fraction
 // bits (exact: its mantissa has 24 bits and z0 >= 1).
@@ -197,7 +200,7 @@ __device__ __forceinline__ Fx<0> rcp_above1(Fx<4> x)
     return {((long long)r0 << 31) + wide(r0, hh) + (wide(r0, hl) >> 31)};
 }
 
-// 1/x as Fx<L> for x in [2^-L, 1), in the same way (30 - L fraction bits of the estimate)
+// 1/x as Fx<L> for x in (2^-L, 1) as in_window admits it, in the same way (30 - L fraction bits of the estimate)
 template <int L>
 __device__ __forceinline__ Fx<L> rcp_below1(Fx<0> x)
 {
