@@ -231,15 +231,17 @@ rok_status build_geometry(rok_ctx *c)
                             &c->G.inv_vol};
     for (int k = 0; k < 15; ++k)
         if ((s = up(*src[k], dst[k])) != ROK_OK) return s;
-    if (!c->strict && c->C.fx.ok) {   // the FMA build's stencil reads the face metrics in fixed point
-        FixedMetric *p = nullptr;
-        if (cudaMalloc(&p, (nfi + nfj) * sizeof(FixedMetric)) != cudaSuccess) return ROK_ERR_NOMEM;
-        c->geo_bufs.push_back(reinterpret_cast<double *>(p));
+    if (!c->strict && c->C.viscous) {
+        double *p = nullptr;
+        if (cudaMalloc(&p, kViscCoefs * (nfi + nfj) * sizeof(double)) != cudaSuccess) return ROK_ERR_NOMEM;
+        c->geo_bufs.push_back(p);
+        // on the copies' stream, finished before any other stream reads
         const CurvGeom &G = c->G;
-        CU(fast::launch_fixed_metrics(G.in_x, G.in_y, G.il, G.ic0, G.ic1, G.ic2, G.ic3, nfi, p, c->stream));
-        CU(fast::launch_fixed_metrics(G.jn_x, G.jn_y, G.jl, G.jc0, G.jc1, G.jc2, G.jc3, nfj, p + nfi, c->stream));
-        c->G.fi = p;
-        c->G.fj = p + nfi;
+        CU(fast::launch_visc_coefs(c->C, G.in_x, G.in_y, G.ic0, G.ic1, G.ic2, G.ic3, nfi, p, cudaStreamLegacy));
+        CU(fast::launch_visc_coefs(c->C, G.jn_x, G.jn_y, G.jc0, G.jc1, G.jc2, G.jc3, nfj, p + kViscCoefs * nfi,
+                                   cudaStreamLegacy));
+        c->G.iv = p;
+        c->G.jv = p + kViscCoefs * nfi;
     }
     const double *tmp;
     if ((s = up(six, &tmp)) != ROK_OK) return s; c->cfl_six = const_cast<double *>(tmp); c->geo_bufs.pop_back();
@@ -247,6 +249,7 @@ rok_status build_geometry(rok_ctx *c)
     if ((s = up(sjx, &tmp)) != ROK_OK) return s; c->cfl_sjx = const_cast<double *>(tmp); c->geo_bufs.pop_back();
     if ((s = up(sjy, &tmp)) != ROK_OK) return s; c->cfl_sjy = const_cast<double *>(tmp); c->geo_bufs.pop_back();
     if ((s = up(vol, &tmp)) != ROK_OK) return s; c->cfl_vol = const_cast<double *>(tmp); c->geo_bufs.pop_back();
+    CU(cudaStreamSynchronize(cudaStreamLegacy));   // pageable copies may still be on their way
     return ROK_OK;
 }
 

@@ -396,7 +396,6 @@ rok_status rok_batch_init(rok_batch **out, const rok_problem_desc *descs, int co
         I.hrdy = 0.5 * I.rdy;
         if (d.kind == ROK_NS2D)
             face_coefs(I.mu, d.sutherland_s > 0.0, d.gamma / ((d.gamma - 1.0) * d.prandtl), I.rdx, I.rdy, I.vk);
-        set_fixed_visc(I.vk, d.sutherland_s > 0.0 ? I.mu : 1.0, I.fxv);
         off += (size_t)I.nchunks * kChunk;
         chunk += I.nchunks;
         for (int c = 0; c < I.nchunks; ++c) chunk_inst.push_back(k);

@@ -27,13 +27,6 @@ struct Fx {
 
 constexpr long long kOne62 = 1ll << 62;
 
-// the constant x (|x| < 2^S) as Fx<S>, at compile time
-template <int S>
-__device__ __forceinline__ constexpr Fx<S> fixed_const(double x)
-{
-    return {(long long)(x * (double)(1ll << (62 - S)))};
-}
-
 // limbs of v = hi 2^31 + lo, 0 <= lo < 2^31
 __device__ __forceinline__ int limb_hi(long long v) { return (int)(v >> 31); }
 __device__ __forceinline__ int limb_lo(long long v) { return (int)v & 0x7fffffff; }
@@ -76,13 +69,6 @@ __device__ __forceinline__ Fx<S> to(Fx<SA> a)
     if (S >= SA) return {a.v >> (S >= SA ? S - SA : 0)};
     return {a.v << (S < SA ? SA - S : 0)};
 }
-// half the number in the same scale
-template <int S>
-__device__ __forceinline__ Fx<S> half_of(Fx<S> a)
-{
-    return {a.v >> 1};
-}
-
 template <int S>
 __device__ __forceinline__ Fx<S> operator+(Fx<S> a, Fx<S> b) { return {a.v + b.v}; }
 template <int S>
@@ -95,9 +81,6 @@ __device__ __forceinline__ Fx<S> abs_of(Fx<S> a)
     const long long m = a.v >> 63;
     return {(a.v ^ m) - m};
 }
-template <int S>
-__device__ __forceinline__ Fx<S> pick(bool c, Fx<S> a, Fx<S> b) { return {c ? a.v : b.v}; }
-
 __device__ __forceinline__ int hi_word(long long v) { return (int)(v >> 32); }
 
 // |x| >= 2^(S - LOG) (on the high word: to 2^-30 of the scale)
@@ -117,18 +100,6 @@ __device__ __forceinline__ bool in_window(Fx<S> a)
     return (unsigned)hi_word(a.v) - lo < (1u << 30) - lo;
 }
 
-// mul with a test that the result is below 2^(S - LOG) in magnitude, made on
-// the product of the high limbs (so that a result that would wrap is caught)
-template <int S, int LOG, int SA, int SB>
-__device__ __forceinline__ Fx<S> mul_below(Fx<SA> a, Fx<SB> b, bool &bad)
-{
-    constexpr int K = SA + SB - S;
-    static_assert(K > 0 && K + LOG <= 28, "the bound needs bits of the high product's high word");
-    const Fx<0> h = {wide(limb_hi(a.v), limb_hi(b.v))};
-    if (outside<K + LOG>(h)) bad = true;
-    return {mul62k<K>(a.v, b.v)};
-}
-
 // the number rounded to 53 significant bits (ties upwards), as binary64 holds it
 template <int S>
 __device__ __forceinline__ Fx<S> round53(Fx<S> a)
@@ -140,26 +111,9 @@ __device__ __forceinline__ Fx<S> round53(Fx<S> a)
     return {(long long)((r & 0xffffffff00000000ull) | ((unsigned)r & (0u - one)))};
 }
 
-// x 2^-e as Fx<S>; low bits beyond 2^(S - 62) are dropped (towards zero).
-// bad is set for |x| 2^-e >= 2^S, infinities and NaN.
-template <int S>
-__device__ __forceinline__ Fx<S> from_double(double x, int e, bool &bad)
-{
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int ex = (int)((hi >> 20) & 0x7ffu);
-    const unsigned mh = ex ? (hi & 0xfffffu) | 0x100000u : hi & 0xfffffu;
-    const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 9;   // top bit 61 where normal
-    const int n = 1022 + S + e - ex;
-    if (n < 0) bad = true;
-    unsigned long long r;
-    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(n < 0 ? 64 : n));   // 64 and more: zero
-    const long long s = (long long)((int)hi >> 31);
-    return {((long long)r ^ s) - s};
-}
-
-// z = 1/sqrt(x) as Fx<L/2> and s = sqrt(x) as Fx<0> for x in [2^-L, 1), L = 6
-// or 8, the lower end excluded (in_window): the hardware's binary32 estimate z0 (relative error about 2^-22) and
-// one third-order step, with e = 1 - x z0^2: z = z0 (1 + e/2 + 3 e^2/8)
+// z = 1/sqrt(x) as Fx<L/2> and s = sqrt(x) as Fx<0> for x in (2^-L, 1) as in_window
+// admits it, L = 6 or 8: the hardware's binary32 estimate z0 (relative error about
+// 2^-22) and one third-order step, with e = 1 - x z0^2: z = z0 (1 + e/2 + 3 e^2/8)
 // (Householder's method), error O(e^3) below the last bit.  z0 has FB fraction
 // bits (exact: its mantissa has 24 bits and z0 >= 1).
 template <int L>

@@ -31,16 +31,7 @@ struct FixedConsts {
     long long efix, hfix;      // efix (0), 1 / (2 efix) (3)
     long long c_lo, c_hi;      // 0
     long long gg, gm1;         // 3, 0
-    long long suth_s, suth_1s; // s / 4 (0), 1 + s (1)
-    long long g_inf;           // mu / mu_ref of the free stream (2; negative: out of range)
-    long long itref;           // 1 / t_ref = itref 2^(itref_e - 62), mantissa in [1/2, 1)
-    int itref_e;
-};
-
-// Viscous coefficients vk as mantissas below 1/2 with one exponent: vk = k 2^(e - 62)
-struct FixedVisc {
-    long long k[2][5];
-    int e;
+    long long suth_s, suth_1s; // s / 8 (0), 1 + s (1)
 };
 
 // Constants of the finite-volume residual (Sec. 3.2).  Every derived constant is
@@ -66,7 +57,6 @@ struct StencilConsts {
     double vk[2][5];
     double vc[4];
     FixedConsts fx;
-    FixedVisc fxv;
     double efix_k;             // (1 - efix) / (1 + efix): c~ efix_k >= |u~| <=> c~ - |u~| >= efix (|u~| + c~)
 };
 
@@ -93,23 +83,6 @@ inline void face_coefs(double mu, bool sutherland, double kfac, double rdx, doub
     }
 }
 
-// the mantissas of factor vk (nothing finite: an exponent no state's units reach)
-inline void set_fixed_visc(const double vk[2][5], double factor, FixedVisc &V)
-{
-    double m = 0.0;
-    for (int d = 0; d < 2; ++d)
-        for (int q = 0; q < 5; ++q) {
-            const double a = fabs(factor * vk[d][q]);
-            m = a > m || !(a == a) ? a : m;
-        }
-    const bool zero = m == 0.0, finite = m < 1e300 && m > 1e-300;
-    int x = 0;
-    if (finite) frexp(m, &x);
-    V.e = zero ? -2000 : (finite ? x + 1 : 1 << 20);
-    for (int d = 0; d < 2; ++d)
-        for (int q = 0; q < 5; ++q) V.k[d][q] = finite ? (long long)ldexp(factor * vk[d][q], 62 - V.e) : 0;
-}
-
 // the fixed-point constants from the gas model and scheme constants (gm1, gg, c_lo,
 // c_hi, efix, inv_tref, suth_s)
 template <class Consts>
@@ -119,12 +92,12 @@ inline void set_fixed_consts(Consts &C)
     F = FixedConsts{};
     F.ok = C.gm1 >= 0.2 && C.gm1 < 1.0 && C.gg <= 6.0 && fabs(C.c_lo) < 1.0 && fabs(C.c_hi) < 1.0 && C.efix >= 0.0 &&
            C.efix < 1.0;
-    if (C.sutherland) F.ok = F.ok && C.suth_s > 0.0 && C.suth_s < 1.0 && C.inv_tref > 1e-300 && C.inv_tref < 1e300;
+    if (C.sutherland) F.ok = F.ok && C.suth_s > 0.0 && C.suth_s < 1.0;
     if (!F.ok) return;
     const double lo = (1.0 - C.efix) / (1.0 + C.efix), hi = (1.0 + C.efix) / (1.0 - C.efix);
     F.m_lo = (int)ldexp(lo, 26);
     F.m_hi = (int)ceil(ldexp(hi < 31.0 ? hi : 31.0, 26));
-    F.fix_ok = C.efix > 0.0625 && C.efix <= 1.0 / 3.0;
+    F.fix_ok = C.efix > 0.0625 && C.efix <= 0.32;
     F.efix = (long long)ldexp(C.efix, 62);
     F.hfix = F.fix_ok ? (long long)ldexp(0.5 / C.efix, 59) : 0;
     F.c_lo = (long long)ldexp(C.c_lo, 62);
@@ -132,11 +105,8 @@ inline void set_fixed_consts(Consts &C)
     F.gg = (long long)ldexp(C.gg, 59);
     F.gm1 = (long long)ldexp(C.gm1, 62);
     if (C.sutherland) {
-        F.suth_s = (long long)ldexp(C.suth_s, 60);
+        F.suth_s = (long long)ldexp(C.suth_s, 59);
         F.suth_1s = (long long)ldexp(1.0 + C.suth_s, 61);
-        const double g = C.prim_inf[5] / C.mu;
-        F.g_inf = g >= 0.0 && g < 2.0 ? (long long)ldexp(g, 60) : -1;
-        F.itref = (long long)ldexp(frexp(C.inv_tref, &F.itref_e), 62);
     }
 }
 
@@ -155,27 +125,19 @@ inline void set_fast_consts(StencilConsts &C)
     C.vc[2] = m;
     C.vc[3] = m * C.kfac;
     set_fixed_consts(C);
-    const double curv[2][5] = {{C.vc[0], C.vc[1], C.vc[2], C.vc[3], 0.0}, {}};
-    set_fixed_visc(C.rdx > 0.0 ? C.vk : curv, C.sutherland ? C.mu : 1.0, C.fxv);   // rdx: 0 on curvilinear grids
 }
-
-// Fixed-point metrics of one face (64 bytes, read as four 16-byte words): the
-// unit normal, the diamond coefficients (c1, c3: a quarter, for four-cell
-// differences) as mantissas, c = mantissa 2^(e - 62), and half the face length
-struct alignas(16) FixedMetric {
-    long long nx, ny, c0, c1, c2, c3;
-    double hlen;
-    long long e;
-};
 
 // Face metrics of a curvilinear grid (device arrays).
 struct CurvGeom {
-    const FixedMetric *fi, *fj;   // FMA build: the faces' fixed-point metrics (same indices)
     // i-faces: (nx+1) * ny, index j*(nx+1)+i ; j-faces: nx * (ny+1), index j*nx+i
     const double *in_x, *in_y, *il, *ic0, *ic1, *ic2, *ic3;
     const double *jn_x, *jn_y, *jl, *jc0, *jc1, *jc2, *jc3;
     const double *inv_vol;     // nx * ny
+    // FMA build, viscous: kViscCoefs coefficients a face (launch_visc_coefs), array q of
+    // n faces at q * n
+    const double *iv, *jv;
 };
+constexpr int kViscCoefs = 10;
 
 // Inputs and epilogue of one stencil launch:
 //   state = base + sum_t c_t add_t [+ cf addf]     (c_t from coef or *coef_dev;
@@ -216,7 +178,6 @@ struct BatchInst {
     int chunk0, nchunks;       // first 2048-entry chunk and chunk count P_k
     double rdx, rdy, q_rdx, q_rdy, mu;
     double hrdx, hrdy, vk[2][5];   // FMA-build constants (face_coefs)
-    FixedVisc fxv;
 };
 
 // Tile table of one batched stencil launch (device arrays): CTA b computes tile
@@ -236,10 +197,9 @@ inline int shape_ty(int s) { return s == kShape16x16 ? 16 : (s == kShape64x4 ? 4
 
 // stencil launchers, one set per rounding mode (separate translation units)
 namespace fast {
-// FMA build: the fixed-point metrics of n faces from their device arrays
-cudaError_t launch_fixed_metrics(const double *nx, const double *ny, const double *len, const double *c0,
-                                 const double *c1, const double *c2, const double *c3, size_t n, FixedMetric *out,
-                                 cudaStream_t s);
+// the viscous coefficients of n faces (FMA build) from their metrics
+cudaError_t launch_visc_coefs(const StencilConsts &c, const double *nx, const double *ny, const double *c0,
+                              const double *c1, const double *c2, const double *c3, size_t n, double *out, cudaStream_t s);
 cudaError_t launch_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s);
 cudaError_t launch_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s);
 cudaError_t launch_lorenz(const StencilConsts &c, const StencilIO &io, int n, cudaStream_t s);

@@ -37,7 +37,6 @@ namespace ROK_NS {
 template <int TXv, int TYv, int NTv = TXv * TYv>
 struct Shape {
     static constexpr int TX = TXv, TY = TYv, NT = NTv, EW = TXv + 4, EH = TYv + 4;
-
 };
 using Shape32x8 = Shape<32, 8>;
 using CurvShape = Shape<16, 16>;
@@ -1371,7 +1370,7 @@ static cudaError_t launch_cart_t(const StencilConsts &c, const StencilIO &io, cu
 template <bool V, bool SU, class SH>
 static cudaError_t launch_fixed_tiles(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
-    const size_t smem = FixedSmem<SU, SH>::bytes;
+    const size_t smem = FixedSmem<V, SU, SH>::bytes;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(fixed_cart_kernel<V, SU, SH, kFixedMinB>,
@@ -1384,32 +1383,17 @@ static cudaError_t launch_fixed_tiles(const StencilConsts &c, const StencilIO &i
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256)
-    fixed_metrics_kernel(const double *nx, const double *ny, const double *len, const double *c0, const double *c1,
-                         const double *c2, const double *c3, size_t n, FixedMetric *out)
+cudaError_t launch_visc_coefs(const StencilConsts &c, const double *nx, const double *ny, const double *c0,
+                              const double *c1, const double *c2, const double *c3, size_t n, double *out, cudaStream_t s)
 {
-    const size_t f = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (f < n) out[f] = fixed_metric(nx[f], ny[f], len[f], c0[f], c1[f], c2[f], c3[f]);
-}
-
-cudaError_t launch_fixed_metrics(const double *nx, const double *ny, const double *len, const double *c0,
-                                 const double *c1, const double *c2, const double *c3, size_t n, FixedMetric *out,
-                                 cudaStream_t s)
-{
-    fixed_metrics_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nx, ny, len, c0, c1, c2, c3, n, out);
+    visc_coefs_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c, nx, ny, c0, c1, c2, c3, n, out);
     return cudaGetLastError();
 }
 
-// Curvilinear faces take the small tile at every size: its one round of eight
-// face batches runs the long face code once per CTA (the larger tiles' warps
-// drift apart in it and miss the instruction cache).  FD-JVP with Sutherland's
-// law, us, 16 x 7 / 16 x 16 / 32 x 15: 256 x 128 14.9 / 21.1 / 37.6; 512 x 256
-// 45.0 / 52.5 / 50.8; 1024 x 512 177 / 178 / 182.
-template <bool V, bool SU>
-static cudaError_t launch_fixed_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
+template <bool V, bool SU, class SH>
+static cudaError_t launch_fixed_curv_tiles(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
 {
-    typedef FixedShapeS SH;
-    const size_t smem = FixedSmem<SU, SH>::bytes;
+    const size_t smem = FixedSmem<V, SU, SH>::bytes;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(fixed_curv_kernel<V, SU, SH, kFixedMinB>,
@@ -1422,19 +1406,31 @@ static cudaError_t launch_fixed_curv(const StencilConsts &c, const CurvGeom &g, 
     return cudaGetLastError();
 }
 
-// The tile by the grid's size (the bits do not depend on it).  FD-JVP, viscous,
-// us a launch (graph nodes), 16 x 7 / 16 x 16 / 32 x 15: 128^2 8.8 / 15.3 / 23.9
-// (below one CTA per SM the smallest chain of rounds wins); 256^2 20.3 / 21.3 /
-// 24.2; 384^2 37.9 / 37.1 / 44.5; 512^2 63.2 / 59.9 / 59.6; 768^2 138 / 131 /
-// 122; 1024^2 267 / 231 / 212 (32 x 15 loads 1.43 cells a cell where 16 x 16
-// loads 1.56 and 16 x 7 1.96, but wants three waves of 3 CTAs per SM).
+// The tiles by the grid's size (the bits do not depend on it): the smallest while its
+// CTAs make one wave of three per SM (152 SMs), where the chain of face rounds in a tile
+// is the time; 32 x 15 from 7.5 tiles an SM on (it loads 1.43 cells a cell where
+// 16 x 16 loads 1.56 and 16 x 7 1.96).  Residual, us a launch (graph nodes), 16 x 7 / 16 x 16 / 32 x 15,
+// Navier-Stokes: 128^2 9.3 / 16.2 / 27.4; 192^2 17.7 / 16.3 / 27.5; 224^2 17.8 / 24.5 / 27.6; 256^2
+// 24.4 / 24.6 / 27.7; 512^2 79.1 / 72.9 / 77.0; 768^2 165 / 157 / 154; 1024^2 292 / 269 / 254; Euler: 128^2
+// 7.7 / 14.3 / 22.2; 256^2 20.2 / 21.5 / 22.3; 512^2 59.7 / 58.5 / 62.0; 1024^2 208 / 198 / 195.
 template <bool V, bool SU>
 static cudaError_t launch_fixed_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
     auto tiles = [&](int tx, int ty) { return (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty); };
+    if (tiles(16, 7) <= 456) return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
     if (tiles(32, 15) >= 1140) return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
-    if (tiles(16, 16) > 456) return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
-    return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
+    return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
+}
+
+// Curvilinear grids: the small tile up to six 16 x 16 tiles an SM.  Residual with
+// Sutherland's law, us, 16 x 7 / 16 x 16 / 32 x 15: 256 x 128 18.3 / 21.6 / 39.5; 384 x 192
+// 38.2 / 32.1 / 51.9; 512 x 256 57.0 / 60.4 / 54.5; 768 x 384 121 / 114 / 121; 1024 x 512 210 / 193 / 200.
+template <bool V, bool SU>
+static cudaError_t launch_fixed_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
+{
+    const long long tiles = (long long)((c.nx + 15) / 16) * ((c.ny + 15) / 16);
+    if (tiles > 912) return launch_fixed_curv_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, g, io, s);
+    return launch_fixed_curv_tiles<V, SU, FixedShapeS>(c, g, io, s);
 }
 #endif
 
@@ -1479,7 +1475,7 @@ static cudaError_t launch_cart_batch_t(const StencilConsts &c, const StencilIO &
 #ifdef ROK_STENCIL_FAST
     if (c.fx.ok) {
         typedef FixedShape<SH> FS;
-        const size_t smem = FixedSmem<SU, FS>::bytes;
+        const size_t smem = FixedSmem<V, SU, FS>::bytes;
         static bool attr_set = false;
         if (!attr_set) {
             cudaError_t e = cudaFuncSetAttribute(fixed_batch_kernel<V, SU, FS, kFixedMinB>,
@@ -1531,7 +1527,7 @@ cudaError_t launch_curv(const StencilConsts &c, const CurvGeom &g, const Stencil
 {
     const bool dual = io.dir || io.dirf;
 #ifdef ROK_STENCIL_FAST
-    if (!dual && c.fx.ok && g.fi) {
+    if (!dual && c.fx.ok) {
         if (!c.viscous) return launch_fixed_curv<false, false>(c, g, io, s);
         return c.sutherland ? launch_fixed_curv<true, true>(c, g, io, s) : launch_fixed_curv<true, false>(c, g, io, s);
     }
