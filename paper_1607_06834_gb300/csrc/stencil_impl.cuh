@@ -1418,7 +1418,8 @@ static cudaError_t launch_fixed_cart(const StencilConsts &c, const StencilIO &io
 {
     auto tiles = [&](int tx, int ty) { return (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty); };
     if (tiles(16, 7) <= 456) return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
-    if (tiles(32, 15) >= 1140) return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
+    if (tiles(32, 15) >= 1140 && c.ny <= 15 * 65535)   // taller grids: 16 rows a tile, as many as a launch holds
+        return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
     return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
 }
 
