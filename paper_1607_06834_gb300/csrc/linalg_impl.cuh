@@ -1724,20 +1724,11 @@ __global__ void __launch_bounds__(RT) gs_normalize_kernel(const double *__restri
     store8(v, e0, n, x);
 }
 
-static int device_sms()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 0;
-    return sms;
-}
-
 static cudaError_t gs_column(double *w, double *V, size_t ldv, size_t n, int j, int next, double *part, StepState *st,
                              long long *launches, cudaStream_t s)
 {
     const int chunks = reduction_blocks(n);
-    const int sms = device_sms();
+    const int sms = sm_count();
     if (sms <= 0) return cudaErrorUnknown;
     const int G = chunks < kGsCtas * sms ? chunks : kGsCtas * sms;
     const int blocks = (j + 4) / 4;
@@ -2822,13 +2813,7 @@ static cudaError_t multidot(const double *F, const void *V, int fp32, size_t ldv
 {
 #ifdef ROK_LINALG_FAST
     {   // even split, one CTA per SM (the strict build keeps the oracle's chunks)
-        static int sms = 0;
-        if (sms == 0) {
-            int dev = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess ||
-                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                sms = -1;
-        }
+        const int sms = sm_count();
         int G = sms > 0 && P > sms ? sms : P;
         auto range = [&] { return ((n + G - 1) / G + 3) & ~(size_t)3; };
         while (G > 1 && (size_t)(G - 1) * range() >= n) --G;   // every CTA has entries

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "rok.h"
 
 namespace rok {
@@ -20,6 +22,37 @@ enum : int {
     kStatusTimeout = 4,    // a bounded device wait (arrival counter) gave up
 };
 
+
+// What the launchers ask of a device, kept once per device (at most 64; others are asked
+// every time).  Asking or setting twice is harmless, so threads need no lock.
+constexpr int kCachedDevices = 64;
+
+// SMs of the current device, 0 on an error
+inline int sm_count()
+{
+    static std::atomic<int> known[kCachedDevices];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const bool cached = dev < kCachedDevices;
+    if (cached && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (cached) known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// allows a kernel `bytes' of dynamic shared memory on the current device; done: one bit
+// a device, of this kernel
+inline cudaError_t allow_shared(std::atomic<uint64_t> &done, const void *kernel, size_t bytes)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < kCachedDevices ? 1ull << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 
 // Constants of the fixed-point stencil (FMA build, stencil_fixed.cuh): numbers
 // x 2^(62 - S), S the scale in the name's comment, and the bounds of the Mach

@@ -1354,13 +1354,8 @@ static cudaError_t launch_cart_t(const StencilConsts &c, const StencilIO &io, cu
     constexpr int MINB = sizeof(S) == sizeof(double) ? 3 : 1;
     const size_t smem = sizeof(Tile<S, CartShape>) + sizeof(Faces<S, CartShape>) + sizeof(Diffs<S, CartShape>) +
                         pair_sums_bytes<V, S, CartShape>();
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(cart_kernel<V, SU, S, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> allowed;
+    if (const cudaError_t e = allow_shared(allowed, (const void *)cart_kernel<V, SU, S, MINB>, smem)) return e;
     dim3 grid((c.nx + CartShape::TX - 1) / CartShape::TX, (c.ny + CartShape::TY - 1) / CartShape::TY);
     cart_kernel<V, SU, S, MINB><<<grid, CartShape::NT, smem, s>>>(c, io);
     return cudaGetLastError();
@@ -1371,13 +1366,8 @@ template <bool V, bool SU, class SH>
 static cudaError_t launch_fixed_tiles(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
     const size_t smem = FixedSmem<V, SU, SH>::bytes;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(fixed_cart_kernel<V, SU, SH, kFixedMinB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> allowed;
+    if (const cudaError_t e = allow_shared(allowed, (const void *)fixed_cart_kernel<V, SU, SH, kFixedMinB>, smem)) return e;
     dim3 grid((c.nx + SH::TX - 1) / SH::TX, (c.ny + SH::TY - 1) / SH::TY);
     fixed_cart_kernel<V, SU, SH, kFixedMinB><<<grid, SH::NT, smem, s>>>(c, io);
     return cudaGetLastError();
@@ -1394,31 +1384,28 @@ template <bool V, bool SU, class SH>
 static cudaError_t launch_fixed_curv_tiles(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
 {
     const size_t smem = FixedSmem<V, SU, SH>::bytes;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(fixed_curv_kernel<V, SU, SH, kFixedMinB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> allowed;
+    if (const cudaError_t e = allow_shared(allowed, (const void *)fixed_curv_kernel<V, SU, SH, kFixedMinB>, smem)) return e;
     dim3 grid((c.nx + SH::TX - 1) / SH::TX, (c.ny + SH::TY - 1) / SH::TY);
     fixed_curv_kernel<V, SU, SH, kFixedMinB><<<grid, SH::NT, smem, s>>>(c, g, io);
     return cudaGetLastError();
 }
 
 // The tiles by the grid's size (the bits do not depend on it): the smallest while its
-// CTAs make one wave of three per SM (152 SMs), where the chain of face rounds in a tile
+// CTAs make one wave of three per SM, where the chain of face rounds in a tile
 // is the time; 32 x 15 from 7.5 tiles an SM on (it loads 1.43 cells a cell where
-// 16 x 16 loads 1.56 and 16 x 7 1.96).  Residual, us a launch (graph nodes), 16 x 7 / 16 x 16 / 32 x 15,
-// Navier-Stokes: 128^2 9.3 / 16.2 / 27.4; 192^2 17.7 / 16.3 / 27.5; 224^2 17.8 / 24.5 / 27.6; 256^2
+// 16 x 16 loads 1.56 and 16 x 7 1.96).  Residual on 152 SMs, us a launch (graph nodes), 16 x 7 / 16 x 16 /
+// 32 x 15, Navier-Stokes: 128^2 9.3 / 16.2 / 27.4; 192^2 17.7 / 16.3 / 27.5; 224^2 17.8 / 24.5 / 27.6; 256^2
 // 24.4 / 24.6 / 27.7; 512^2 79.1 / 72.9 / 77.0; 768^2 165 / 157 / 154; 1024^2 292 / 269 / 254; Euler: 128^2
 // 7.7 / 14.3 / 22.2; 256^2 20.2 / 21.5 / 22.3; 512^2 59.7 / 58.5 / 62.0; 1024^2 208 / 198 / 195.
 template <bool V, bool SU>
 static cudaError_t launch_fixed_cart(const StencilConsts &c, const StencilIO &io, cudaStream_t s)
 {
     auto tiles = [&](int tx, int ty) { return (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty); };
-    if (tiles(16, 7) <= 456) return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
-    if (tiles(32, 15) >= 1140 && c.ny <= 15 * 65535)   // taller grids: 16 rows a tile, as many as a launch holds
+    const int sms = sm_count();
+    if (sms <= 0) return cudaErrorUnknown;
+    if (tiles(16, 7) <= 3 * sms) return launch_fixed_tiles<V, SU, FixedShapeS>(c, io, s);
+    if (2 * tiles(32, 15) >= 15 * sms && c.ny <= 15 * 65535)   // taller grids: 16 rows a tile, as many as a launch holds
         return launch_fixed_tiles<V, SU, FixedShapeL>(c, io, s);
     return launch_fixed_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, io, s);
 }
@@ -1430,7 +1417,9 @@ template <bool V, bool SU>
 static cudaError_t launch_fixed_curv(const StencilConsts &c, const CurvGeom &g, const StencilIO &io, cudaStream_t s)
 {
     const long long tiles = (long long)((c.nx + 15) / 16) * ((c.ny + 15) / 16);
-    if (tiles > 912) return launch_fixed_curv_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, g, io, s);
+    const int sms = sm_count();
+    if (sms <= 0) return cudaErrorUnknown;
+    if (tiles > 6 * sms) return launch_fixed_curv_tiles<V, SU, FixedShape<Shape<16, 16>>>(c, g, io, s);
     return launch_fixed_curv_tiles<V, SU, FixedShapeS>(c, g, io, s);
 }
 #endif
@@ -1440,13 +1429,8 @@ static cudaError_t launch_curv_t(const StencilConsts &c, const CurvGeom &g, cons
 {
     constexpr int MINB = sizeof(S) == sizeof(double) ? 3 : 1;
     const size_t smem = sizeof(Tile<S>) + sizeof(Faces<S>) + sizeof(Diffs<S>);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(curv_kernel<V, SU, S, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> allowed;
+    if (const cudaError_t e = allow_shared(allowed, (const void *)curv_kernel<V, SU, S, MINB>, smem)) return e;
     dim3 grid((c.nx + TX - 1) / TX, (c.ny + TY - 1) / TY);
     curv_kernel<V, SU, S, MINB><<<grid, NT, smem, s>>>(c, g, io);
     return cudaGetLastError();
@@ -1477,26 +1461,16 @@ static cudaError_t launch_cart_batch_t(const StencilConsts &c, const StencilIO &
     if (c.fx.ok) {
         typedef FixedShape<SH> FS;
         const size_t smem = FixedSmem<V, SU, FS>::bytes;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(fixed_batch_kernel<V, SU, FS, kFixedMinB>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            attr_set = true;
-        }
+        static std::atomic<uint64_t> allowed;
+        if (const cudaError_t e = allow_shared(allowed, (const void *)fixed_batch_kernel<V, SU, FS, kFixedMinB>, smem)) return e;
         fixed_batch_kernel<V, SU, FS, kFixedMinB><<<ntiles, FS::NT, smem, s>>>(c, io, bt);
         return cudaGetLastError();
     }
 #endif
     const size_t smem = sizeof(Tile<double, SH>) + sizeof(Faces<double, SH>) + sizeof(Diffs<double, SH>) +
                         pair_sums_bytes<V, double, SH>();
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(cart_batch_kernel<V, SU, SH, 3>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> allowed;
+    if (const cudaError_t e = allow_shared(allowed, (const void *)cart_batch_kernel<V, SU, SH, 3>, smem)) return e;
     cart_batch_kernel<V, SU, SH, 3><<<ntiles, SH::NT, smem, s>>>(c, io, bt);
     return cudaGetLastError();
 }
