@@ -553,18 +553,27 @@ rok_status rok_batch_tune(rok_batch *b, const double *y, rok_batch_tuning *out)
             }
         }
     }
-    // vector passes on scratch data: one Arnoldi column (active flags set),
-    // zero partials (h = 0)
+    // Vector passes on one Arnoldi column (active flags set).  The basis vectors are the
+    // state scaled to unit length: ordinary numbers, so that the FMA build's passes
+    // take the sums they take in a step (unwritten memory may be zeros, which they
+    // leave to the binary64 sum).  The strict build's passes get zero partials (h = 0).
     CU(launch_begin_batch(b->st, b->d_h, b->gamma_rok, 1, b->count, b->stream));
-    CU(cudaMemsetAsync(b->pA, 0, 2 * (size_t)b->nchunks * sizeof(double), b->stream));
     const BSeg sg = seg(b);
+    const int nv = b->mmax + 1 < 4 ? b->mmax + 1 : 4;
+    const size_t vbytes = b->total * sizeof(double);
+    CU(b->bops->dot2(y, y, nullptr, nullptr, b->pA, sg, 0, 1, b->stream));
+    CU(b->bops->first_normalize(y, b->V, b->pA, sg, 1, b->stream));
+    for (int q = 1; q < nv; ++q)
+        CU(cudaMemcpyAsync(b->V + (size_t)q * b->total, b->V, vbytes, cudaMemcpyDeviceToDevice, b->stream));
+    CU(cudaMemsetAsync(b->pA, 0, 2 * (size_t)b->nchunks * sizeof(double), b->stream));
     float best_m = -1.0f, best_v = -1.0f;
     for (int q = 0; q < 4; ++q) {
         const int c = kCpcCandidates[q];
         float ms = 0.0f;
+        // every candidate starts from the state (the block's subtraction scales it by up to 3)
+        CU(cudaMemcpyAsync(b->t0, y, vbytes, cudaMemcpyDeviceToDevice, b->stream));
         r = time_ms(b, 3, [&] {
             // FMA build: a full block of the basis, projected on again
-            const int nv = b->mmax + 1 < 4 ? b->mmax + 1 : 4;
             const cudaError_t e =
                 b->bops->gs_pass ? b->bops->gs_pass(b->t0, b->V, b->total, kMaxKrylov - 1, 0, nv, 0, nv, 0, b->pM, sg, c, b->stream)
                                  : b->bops->mgs(b->t0, b->V, b->total, 1, 0, b->pA, b->pB, sg, c, b->stream);
