@@ -7,8 +7,12 @@
 // fixed-point numbers below 2^57 in units set by the operand's largest exponent,
 // and the products of their 29-bit limbs are accumulated exactly.  One rounding
 // to 2^-56 of the largest product and the conversion to binary64 end the sum;
-// the entries themselves lose what lies below 2^-57 of the largest, so the result
-// is closer to the exact sum than a chain of binary64 multiply-adds.  An entry
+// the entries themselves lose (towards zero) what lies below 2^-57 of the largest one of
+// the thread.  So the error is below 2^-52 of (largest |v|) (largest |w|) for 8 terms:
+// smaller than that of a chain of binary64 multiply-adds where the thread's entries
+// are of similar size, as neighbouring cells' are, but relative to the largest
+// product, not to each: a sum whose large entries of one vector all meet small ones
+// of the other keeps fewer digits of its own.  An entry
 // costs 16 integer instructions an operand and four 32 x 32 -> 64 multiply-adds
 // (8 to 10 SM clocks a warp together, against 16 for one FP64 instruction).
 // Operands that are zero, non-finite or far outside the usual exponents are left

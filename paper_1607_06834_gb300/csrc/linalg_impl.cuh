@@ -1274,7 +1274,8 @@ __global__ void __launch_bounds__(kEvenThreads, 1)
             st->active = 0;
             st->meff = j + 1;
         } else {
-            st->H[(j + 1) * kMaxKrylov + j] = hn2 * sh[0];
+            const double hn = hn2 * sh[0];   // and one Newton step: the rounding of the square root
+            st->H[(j + 1) * kMaxKrylov + j] = fma(fma(-hn, hn, hn2), 0.5 * sh[0], hn);
         }
     }
     if (!ok || brk) return;
@@ -1628,7 +1629,8 @@ __device__ __forceinline__ void gs_finish(const GsPass &ps, const double (*tot)[
 {
     if (ps.nn == 0) {
         if (!ps.next) return;
-        const double hn2 = tot[0][0], hn = sqrt(hn2);
+        // the norm and its reciprocal as the column kernel forms them
+        const double hn2 = tot[0][0], rh = rsqrt(hn2), h0 = hn2 * rh, hn = fma(fma(-h0, h0, hn2), 0.5 * rh, h0);
         const double wnorm0 = sqrt(st->gs_ssq + hn2);   // ||J v_j|| (Pythagoras for the orthonormal basis)
         st->wnorm0 = wnorm0;
         if (!(hn > 1e-12 * wnorm0)) {
@@ -1636,7 +1638,7 @@ __device__ __forceinline__ void gs_finish(const GsPass &ps, const double (*tot)[
             st->meff = ps.j + 1;
         } else {
             st->H[(ps.j + 1) * kMaxKrylov + ps.j] = hn;
-            st->gs_rh = 1.0 / hn;
+            st->gs_rh = rh;
         }
         return;
     }
@@ -1935,16 +1937,21 @@ __device__ __forceinline__ long long magnitude_key(double x)
 }
 
 #ifdef ROK_LINALG_FAST
-// 1/x: the hardware estimate and one third-order Newton step (3 FP64
-// instructions; a division takes about ten), the division outside its range
+// 1/x for |x| in [2^-991, 2^992): the hardware estimate and one third-order Newton step
+__device__ __forceinline__ bool reciprocal_range(double x) { return ((unsigned)__double2hiint(x) >> 20 & 0x7ffu) - 32u <= 1982u; }
 __device__ __forceinline__ double reciprocal(double x)
 {
-    const int e = __double2hiint(x) >> 20 & 0x7ff;
-    if (e < 32 || e > 2014) return 1.0 / x;
     double r0;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
     const double d = fma(-x, r0, 1.0);
     return fma(r0, fma(d, d, d), r0);
+}
+// a / d with rd = reciprocal(d): the product corrected by its remainder, which rounds as
+// the division does
+__device__ __forceinline__ double quotient(double a, double d, double rd)
+{
+    const double q = a * rd;
+    return fma(fma(-q, d, a), rd, q);
 }
 #endif
 
@@ -1955,8 +1962,9 @@ __device__ __forceinline__ double reciprocal(double x)
 // division per row, one update per step), so the strict build's factors are those
 // of the plain loops.
 // Bound by the latency of FP64 instructions (64 cycles each on one warp): integer
-// comparisons in the pivot search and, in the FMA build, one reciprocal a step instead
-// of a division a row: 42 -> 22 us at m = 20, 67 -> 35 us at m = 30.
+// comparisons in the pivot search and, in the FMA build, one reciprocal a step and three
+// instructions a row instead of a division (42 -> 23 us at m = 20, 67 -> 37 us at m = 30),
+// which pivots outside the reciprocal's range keep.
 __device__ __forceinline__ void lu_body(StepState *st)
 {
     // the factorisation runs in shared memory; the factors and the pivots are
@@ -2011,11 +2019,12 @@ __device__ __forceinline__ void lu_body(StepState *st)
             break;
         }
 #ifdef ROK_LINALG_FAST
-        const double rd = reciprocal(d);
-        for (int i = k + 1 + tid; i < m; i += nt) A[i * kMaxKrylov + k] = A[i * kMaxKrylov + k] * rd;
-#else
-        for (int i = k + 1 + tid; i < m; i += nt) A[i * kMaxKrylov + k] = A[i * kMaxKrylov + k] / d;
+        if (reciprocal_range(d)) {
+            const double rd = reciprocal(d);
+            for (int i = k + 1 + tid; i < m; i += nt) A[i * kMaxKrylov + k] = quotient(A[i * kMaxKrylov + k], d, rd);
+        } else
 #endif
+            for (int i = k + 1 + tid; i < m; i += nt) A[i * kMaxKrylov + k] = A[i * kMaxKrylov + k] / d;
         __syncthreads();
         const int w = m - k - 1;
         for (int idx = tid; idx < w * w; idx += nt) {
