@@ -130,7 +130,7 @@ inline void set_fixed_consts(Consts &C)
     const double lo = (1.0 - C.efix) / (1.0 + C.efix), hi = (1.0 + C.efix) / (1.0 - C.efix);
     F.m_lo = (int)ldexp(lo, 26);
     F.m_hi = (int)ceil(ldexp(hi < 31.0 ? hi : 31.0, 26));
-    F.fix_ok = C.efix > 0.0625 && C.efix <= 0.32;
+    F.fix_ok = C.efix > 0.0625 && C.efix <= 1.0 / 3.0;
     F.efix = (long long)ldexp(C.efix, 62);
     F.hfix = F.fix_ok ? (long long)ldexp(0.5 / C.efix, 59) : 0;
     F.c_lo = (long long)ldexp(C.c_lo, 62);

@@ -310,7 +310,8 @@ __device__ __forceinline__ void fixed_roe(FixedState L, FixedState R, int kn, in
     const int mh = hi_word(aM.v);
     if (mh >= F.m_lo && mh <= F.m_hi) {   // the fix may act: (ms^2 / delta + delta) / 2 below delta = efix (|M| + 1)
         const Fx<4> d = mul<4>(Fx<0>{F.efix}, mb);
-        const Fx<0> m0 = to<0>(ms);       // below 0.95 for efix up to 0.32 (fix_ok)
+        // below 1 where ms < d, as |M| < 2 there for efix up to 1/3 (fix_ok); h is unused elsewhere
+        const Fx<0> m0 = to<0>(ms);
         const Fx<3> h = {mul<3>(mul<0>(m0, m0), mul<3>(Fx<3>{F.hfix}, rcp_above1(mb))).v + d.v};   // d / 2 as Fx<3>
         if (ms.v < d.v) ms = to<4>(h);
         if (!F.fix_ok) bad = true;
