@@ -549,30 +549,6 @@ __device__ __forceinline__ fx::Fx<0> fixed_normal(double x)
     return {ex >= 1023 ? (__double2hiint(x) < 0 ? -one : one) : fixed_of(x, 1022)};
 }
 
-// ghost rules of one tile cell (global indices gi, gj): the source cell, whether
-// its velocity is mirrored, whether it is the free stream
-__device__ __forceinline__ void curv_source(const StencilConsts &C, int &gi, int &gj, bool &mirror, bool &inf)
-{
-    const int nx = C.nx, ny = C.ny;
-    mirror = inf = false;
-    if (gi < 0 || gi >= nx) {
-        const int b = gi < 0 ? C.bc[0] : C.bc[1];
-        if (b == ROK_BC_PERIODIC) gi = wrapi(gi, nx);
-        else if (b == ROK_BC_WALL) { gi = gi < 0 ? -gi - 1 : 2 * nx - 1 - gi; mirror = !mirror; }
-        else inf = true;
-    }
-    if (!inf && (gj < 0 || gj >= ny)) {
-        const int b = gj < 0 ? C.bc[2] : C.bc[3];
-        if (b == ROK_BC_PERIODIC) gj = wrapi(gj, ny);
-        else if (b == ROK_BC_WALL) { gj = gj < 0 ? -gj - 1 : 2 * ny - 1 - gj; mirror = !mirror; }
-        else inf = true;
-    }
-    // a tile cell past the last valid index of a partial tile may still be out of
-    // range after the rules above; clamp it (its faces are never used)
-    gi = min(max(gi, 0), nx - 1);
-    gj = min(max(gj, 0), ny - 1);
-}
-
 // Viscous coefficients of a curvilinear face.  The doubled stress and heat flux of
 // visc_n2_terms are linear in the differences across (dC) and along (dV, four
 // cells) the face; with the metric terms, the normal and the viscosity multiplied

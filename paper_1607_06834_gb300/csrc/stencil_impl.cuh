@@ -987,6 +987,32 @@ __global__ void __launch_bounds__(CartShape::NT, MINB) cart_kernel(const Stencil
     cart_tile<VISC, SUTH, S, CartShape>(C, io, blockIdx.x * CartShape::TX, blockIdx.y * CartShape::TY, smem_raw);
 }
 
+// Ghost cells of a curvilinear grid: j-ghosts of interior columns first, then
+// i-ghosts of every row (ghost rows included); periodic wraps, a wall mirrors
+// (rho, -u, -v, p), the far field is the free stream.  For one tile cell (global indices
+// gi, gj): the source cell, whether its velocity is mirrored, whether it is the free stream.
+__device__ __forceinline__ void curv_source(const StencilConsts &C, int &gi, int &gj, bool &mirror, bool &inf)
+{
+    const int nx = C.nx, ny = C.ny;
+    mirror = inf = false;
+    if (gi < 0 || gi >= nx) {
+        const int b = gi < 0 ? C.bc[0] : C.bc[1];
+        if (b == ROK_BC_PERIODIC) gi = wrapi(gi, nx);
+        else if (b == ROK_BC_WALL) { gi = gi < 0 ? -gi - 1 : 2 * nx - 1 - gi; mirror = !mirror; }
+        else inf = true;
+    }
+    if (!inf && (gj < 0 || gj >= ny)) {
+        const int b = gj < 0 ? C.bc[2] : C.bc[3];
+        if (b == ROK_BC_PERIODIC) gj = wrapi(gj, ny);
+        else if (b == ROK_BC_WALL) { gj = gj < 0 ? -gj - 1 : 2 * ny - 1 - gj; mirror = !mirror; }
+        else inf = true;
+    }
+    // a tile cell past the last valid index of a partial tile may still be out of
+    // range after the rules above; clamp it (its faces are never used)
+    gi = min(max(gi, 0), nx - 1);
+    gj = min(max(gj, 0), ny - 1);
+}
+
 #ifdef ROK_STENCIL_FAST
 #include "stencil_fixed.cuh"
 #endif
@@ -1026,9 +1052,7 @@ __global__ void __launch_bounds__(SH::NT, MINB) cart_batch_kernel(const StencilC
 }
 
 // ============================== curvilinear grid ===============================
-// Ghost cells follow the boundary rules: j-ghosts of interior columns first,
-// then i-ghosts of every row (ghost rows included); periodic wraps, a wall
-// mirrors (rho, -u, -v, p), the far field is the free stream.
+// (ghost cells: curv_source)
 template <bool VISC, bool SUTH, class S, int MINB>
 __global__ void __launch_bounds__(NT, MINB) curv_kernel(const StencilConsts C, const CurvGeom G, const StencilIO io)
 {
@@ -1048,23 +1072,8 @@ __global__ void __launch_bounds__(NT, MINB) curv_kernel(const StencilConsts C, c
     for (int idx = tid; idx < EW * EH; idx += NT) {
         int lx = idx % EW, ly = idx / EW;
         int gi = i0 + lx - 2, gj = j0 + ly - 2;
-        bool mirror = false, inf = false;
-        if (gi < 0 || gi >= nx) {
-            int b = gi < 0 ? C.bc[0] : C.bc[1];
-            if (b == ROK_BC_PERIODIC) gi = wrapi(gi, nx);
-            else if (b == ROK_BC_WALL) { gi = gi < 0 ? -gi - 1 : 2 * nx - 1 - gi; mirror = !mirror; }
-            else inf = true;
-        }
-        if (!inf && (gj < 0 || gj >= ny)) {
-            int b = gj < 0 ? C.bc[2] : C.bc[3];
-            if (b == ROK_BC_PERIODIC) gj = wrapi(gj, ny);
-            else if (b == ROK_BC_WALL) { gj = gj < 0 ? -gj - 1 : 2 * ny - 1 - gj; mirror = !mirror; }
-            else inf = true;
-        }
-        // a tile cell past the last valid index of a partial tile may still be out
-        // of range after the rules above; clamp it (its faces are never used)
-        gi = min(max(gi, 0), nx - 1);
-        gj = min(max(gj, 0), ny - 1);
+        bool mirror, inf;
+        curv_source(C, gi, gj, mirror, inf);
         if (inf) {
             tl.r[ly][lx] = lift<S>(C.prim_inf[0]);
             tl.u[ly][lx] = lift<S>(mirror ? -C.prim_inf[1] : C.prim_inf[1]);
