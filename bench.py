@@ -41,11 +41,16 @@ FLOPS_RESIDUAL_NS = 390 + 10 + 20
 FLOPS_JVP_NS = FLOPS_RESIDUAL_NS + 8 + 8
 BYTES_RESIDUAL, BYTES_JVP = 64, 128
 
-# DRAM bytes (read + write) of one FD-JVP launch of the Navier-Stokes stencil at
-# 512 x 512, from an ncu capture of this workload (dram__bytes_read.sum +
+# DRAM bytes (read + write) of one FD-JVP launch of the Navier-Stokes stencil (FMA
+# build, fixed_cart_kernel) at 512 x 512, from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum, cold L2): the three inputs y, v, f(y) are read once
-# (25.17 MB algorithmic); the 8.4 MB output stays in L2 within the launch.
-STENCIL_JVP_DRAM_BYTES_512 = 25243136 + 0
+# (25.17 MB algorithmic); most of the 8.4 MB output stays in L2 within the launch.
+STENCIL_JVP_DRAM_BYTES_512 = 25804800 + 753408
+
+# Instructions a cell on the FP64 pipe of that kernel at 512 x 512 (ncu,
+# sm__inst_executed_pipe_fp64.sum x 32 / cells): the pipe that bounds it, as its
+# faces run on the integer pipe and what they leave to FP64 does not.
+FP64_PIPE_RESIDUAL_512, FP64_PIPE_JVP_512 = 850944 * 32 / 512 ** 2, 904192 * 32 / 512 ** 2
 
 
 def _peaks():
@@ -216,6 +221,11 @@ def run_ours(args):
     flops_step = cells * (n_res * FLOPS_RESIDUAL_NS + n_jvp * FLOPS_JVP_NS)
     stencil_ms_per_launch = cnt['stencil_ms'] / max(cnt['stencil_timed'], 1)
     achieved = flops_step / (n_res + n_jvp) / (stencil_ms_per_launch * 1e-3) / 1e12
+    # the FMA build's stencil against the pipe that bounds it: lane-instructions on the
+    # FP64 pipe (counted at 512 x 512) per second; the strict build's against the FMA roof
+    fixed = args.rounding == 'fast'
+    pipe = cells * (n_res * FP64_PIPE_RESIDUAL_512 + n_jvp * FP64_PIPE_JVP_512) / (n_res + n_jvp) / \
+        (stencil_ms_per_launch * 1e-3) / 1e12
     # algorithmic bytes of the average launch: a residual reads q and writes f
     # (64 B per cell), an FD JVP reads y, v, f(y) and writes Jv (128 B per cell)
     bytes_launch = cells * (n_res * BYTES_RESIDUAL + n_jvp * BYTES_JVP) / (n_res + n_jvp)
@@ -348,14 +358,18 @@ def run_ours(args):
                    'launch': 'CUDA-graph replay per step' if args.graph else 'kernel by kernel',
                    'parallelism': 'replicas' if ws > 1 else 'single-gpu'},
         'roofline': {'bound': 'alu', 'kernel': 'residual/JVP stencil (%s<NS>)' % (
-                         'fixed_cart_kernel' if args.rounding == 'fast' else 'cart_kernel'),
-                     'achieved': round(achieved, 4), 'peak': round(fp64_roof, 4), 'unit': 'TFLOP/s',
-                     'frac': round(achieved / fp64_roof, 4),
-                     'traffic': STENCIL_JVP_DRAM_BYTES_512 if N_GRID == 512 else None,
+                         'fixed_cart_kernel' if fixed else 'cart_kernel'),
+                     'achieved': round(pipe if fixed else achieved, 4),
+                     'peak': round(fp64_roof / 2 if fixed else fp64_roof, 4),
+                     'unit': 'T FP64-pipe lane-instructions/s' if fixed else 'TFLOP/s',
+                     'frac': round(2 * pipe / fp64_roof if fixed else achieved / fp64_roof, 4),
+                     'traffic': STENCIL_JVP_DRAM_BYTES_512 if fixed and N_GRID == 512 else None,
                      'traffic_unit': 'bytes per FD-JVP launch (ncu dram read+write)',
                      'algorithmic_bytes_per_launch': round(bytes_launch),
-                     'peak_source': 'FP64 FMA roof = 152 SMs x 2 FMA/clk/SM x 2 flops x measured SM clock; '
-                                    'the kernel runs 62-bit fixed point on the integer pipe, which that roof does not bound',
+                     'peak_source': '152 SMs x 2 FP64 lanes/clk/SM x measured SM clock; the faces run on the integer '
+                                    'pipe, which this does not bound' if fixed else
+                                    'FP64 FMA roof = 152 SMs x 2 FMA/clk/SM x 2 flops x measured SM clock',
+                     'algorithmic_tflops': round(achieved, 4),
                      'fp64_fma_microbenchmark_tflops': round(fp64_peak, 4),
                      'flops_per_cell': {'residual': FLOPS_RESIDUAL_NS, 'jvp': FLOPS_JVP_NS},
                      'stencil_ms_per_launch': round(stencil_ms_per_launch, 5),

@@ -50,8 +50,17 @@ enum { ROK_BC_PERIODIC = 0, ROK_BC_WALL = 1, ROK_BC_FARFIELD = 2 };
 enum { ROK_JVP_FD = 0, ROK_JVP_EXACT = 1 };
 /* ROK_ROUND_STRICT compiles the stencil without multiply-add contraction, so
  * f(y) is the IEEE result of the written-out formulas (bitwise reproducible
- * against a plain CPU evaluation in the same order); ROK_ROUND_FAST lets the
- * compiler contract into FMA (fewer FP64 instructions, last-bit differences). */
+ * against a plain CPU evaluation in the same order).  ROK_ROUND_FAST (default):
+ * primitives, viscous terms and the cell balance in binary64 with FMA, the
+ * reconstruction and Roe's flux of a face in 62-bit fixed point with units (powers
+ * of two) that the face's own four cells set, or in binary64 where the face does
+ * not fit (jumps by more than about 6 across its cells, Mach numbers above 4 to 8).
+ * A face's result depends on its cells alone: not on the tile, the batch or the
+ * rest of the grid.  Rounding errors are those of binary64, by component and at
+ * any scale of density, pressure and velocity (rms against long double 0.4 to 1.3
+ * times the strict build's); the results differ from it in the last bits.  Problems
+ * with gamma outside (1.2, 2), entropy_fix >= 1 or sutherland_s >= 1 take a binary64
+ * kernel. */
 enum { ROK_ROUND_FAST = 0, ROK_ROUND_STRICT = 1 };
 /* Krylov basis of the ROK step: binary64, or binary32 storage with binary32
  * Gram-Schmidt (the mixed-precision form; the state, the finite-difference
