@@ -231,7 +231,7 @@ rok_status build_geometry(rok_ctx *c)
                             &c->G.inv_vol};
     for (int k = 0; k < 15; ++k)
         if ((s = up(*src[k], dst[k])) != ROK_OK) return s;
-    if (!c->strict && c->C.viscous) {
+    if (!c->strict && c->C.viscous && c->C.fx.ok) {
         double *p = nullptr;
         if (cudaMalloc(&p, kViscCoefs * (nfi + nfj) * sizeof(double)) != cudaSuccess) return ROK_ERR_NOMEM;
         c->geo_bufs.push_back(p);
